@@ -692,6 +692,11 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p) 
         break;
       }
     }
+    // Peers' thread 0 may still be reading p(x), q(x) from this CTA's slices
+    // (nothing orders the CTAs while children are tried, except a SPEC
+    // rejection): they are rewritten -- the next row, or rejected tokens
+    // zeroed -- only after every CTA has taken its decisions.
+    if (nxt >= 0 || nrej > 0) w.exchange();
     if (nxt >= 0) {
       if (tid == 0) sh.path[plen] = nxt;
       ++plen;
