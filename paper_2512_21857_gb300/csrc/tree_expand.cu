@@ -5,15 +5,24 @@
 // Expand is one launch of F thread-block clusters, one per frontier row; the
 // C <= 8 CTAs of a cluster split the row's vocabulary.  Each CTA stages its
 // share in shared memory with one bulk copy (x / T in fp32, round-to-nearest
-// division).  A first pass keeps each thread's two largest values; the k-th
-// largest of the 32 warp maxima bounds the CTA's top k from below; a second
-// pass sums the exponentials against the CTA's maximum and gathers the few
-// selection keys (value order, then lower index) at or above the bound,
-// which are ranked by counting.  The CTAs' lists go to the cluster's first
+// division).  A first pass keeps each thread's largest value; the k-th
+// largest of the 32 warp maxima (64 half-warp maxima for k > 32) bounds the
+// CTA's top k from below; a second pass sums the exponentials against the
+// CTA's maximum and gathers the few selection keys (value order, then lower
+// index) at or above the bound, which are ranked by counting.  The CTAs' lists go to the cluster's first
 // CTA through distributed shared memory; it ranks them, forms the row's
 // log-sum-exp and writes the row's children (log-probability against it in
 // fp64).  The first CTA of the last row to finish (atomic ticket) ranks the
-// next frontier across all rows.
+// next frontier across all rows.  Every selection of more than 128 keys first
+// bounds them the same way (64 group maxima), so that only about as many as
+// are wanted get ranked.
+//
+// A call is bound by the latency of that chain of phases, not by its bytes
+// (2.1 MB at F = 8, V = 65536: 0.3 us of HBM time).  Back-to-back calls in a
+// graph: 6.5 us at F = 8, V = 65536, k = 8 and 4.8 us at F = 1; 12.6 us at
+// F = 39, V = 16384, k = 39 under guidance.  (With a bound that let half of a
+// CTA's logits through for k > 32, each of them inserted in sorted lists, the
+// last took 221.7 us.)
 #include <cooperative_groups.h>
 
 #include "adt_common.cuh"
@@ -29,7 +38,8 @@ constexpr int kMaxK = 64;
 constexpr int kMaxKeep = 1024;
 constexpr int kMaxCluster = 8;
 constexpr int kValuesPerCta = 2048;     // a CTA per this many logits, up to kMaxCluster per row
-constexpr int kTile = 16384;            // logits staged in shared memory at a time
+constexpr int kTile = 32768;            // logits staged in shared memory at a time
+constexpr int kTileGuided = kTile / 2;  // under guidance (two rows)
 constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr int kCandCap = 1024;          // a CTA's candidate buffer (also the cross-row keys)
 constexpr float kLog2e = 1.44269504088896340736f;
@@ -55,6 +65,7 @@ struct ExpandParams {
   uint64_t* cross_keys;   // [F*k]
   unsigned* all_ticket;   // [1]
   unsigned* err;
+  int tile;               // kTile or kTileGuided
 };
 
 // Entries greater than key in a descending list of n keys.
@@ -145,19 +156,20 @@ struct WarpTopK {
 // aligned and ld is a multiple of 4) in shared memory with one bulk copy
 // (two with guidance: the unconditional row goes to vals_u), waiting with a
 // bound; then forms u + s (c - u) under guidance and divides by the
-// temperature, in place.  Block-wide.
-__device__ bool stage_tile(float* vals, float* vals_u, const float* row, const float* row_u, int t0, int t1,
+// temperature, in place (kPlain: neither).  Block-wide.
+template <bool kPlain>
+__device__ __forceinline__ bool stage_tile(float* vals, float* vals_u, const float* row, const float* row_u, int t0, int t1,
                            const ExpandParams& p, uint64_t* bar, uint32_t& phase) {
   const int n = t1 - t0;
   if (threadIdx.x == 0 && n > 0) {
     const uint32_t bytes = static_cast<uint32_t>((n + 3) / 4 * 16);
-    sm100::mbar_arrive_expect_tx(sm100::smem_addr(bar), row_u ? 2 * bytes : bytes);
+    sm100::mbar_arrive_expect_tx(sm100::smem_addr(bar), !kPlain && row_u ? 2 * bytes : bytes);
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
             sm100::smem_addr(vals)),
         "l"(row + t0), "r"(bytes), "r"(sm100::smem_addr(bar))
         : "memory");
-    if (row_u)
+    if (!kPlain && row_u)
       asm volatile(
           "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
               sm100::smem_addr(vals_u)),
@@ -169,7 +181,7 @@ __device__ bool stage_tile(float* vals, float* vals_u, const float* row, const f
     ok = sm100::mbar_wait_bounded(sm100::smem_addr(bar), phase, kWaitLimit);
     phase ^= 1u;
   }
-  if (row_u || p.use_T) {
+  if (!kPlain && (row_u || p.use_T)) {
     for (int i = threadIdx.x; i < n; i += kThreads) {
       float x = vals[i];
       if (row_u) x = adt::cfg_combine(x, vals_u[i], p.cfg);
@@ -179,20 +191,6 @@ __device__ bool stage_tile(float* vals, float* vals_u, const float* row, const f
   }
   __syncthreads();
   return ok;
-}
-
-// out[rank] = key for the k largest of the n distinct nonzero keys in
-// keys[0..n) (0 entries skipped); out[] zeroed by the caller.  Block-wide:
-// a warp takes a key and its lanes count the keys above it.
-__device__ void rank_select(const uint64_t* keys, int n, int k, uint64_t* out) {
-  const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x >> 5; i < n; i += kWarps) {
-    const uint64_t key = keys[i];
-    if (key == 0ull) continue;
-    int rk = 0;
-    for (int j = 0; j < n; j += 32) rk += __popc(__ballot_sync(adt::kFullMask, j + lane < n && keys[j + lane] > key));
-    if (lane == 0 && rk < k) out[rk] = key;
-  }
 }
 
 // 2^x with the hardware approximation (flush-to-zero); 2^-inf = 0.
@@ -217,29 +215,147 @@ __device__ __forceinline__ float warp_kth_largest(float v, int k, int lane) {
   return __shfl_sync(adt::kFullMask, v, __ffs(m) - 1);
 }
 
-// rank_select for n <= 64 keys: 16 threads per key, each counting the keys
-// above it among four of the others, the counts summed by shuffles within
-// the group; one round of loads instead of a warp per key looping over n.
-__device__ void rank_select64(const uint64_t* keys, int n, int k, uint64_t* out) {
-  static_assert(kThreads == 64 * 16, "16 threads for each of 64 keys");
-  const int i = threadIdx.x >> 4, s = threadIdx.x & 15;
+// out[rank] = key for the k largest of the n (<= kThreads / T) distinct
+// nonzero keys in keys[0..n) (0 entries skipped); out[] zeroed by the caller.
+// Block-wide: T threads per key, each counting the keys above it among every
+// T-th of the others, the counts summed by shuffles within the group.
+template <int T>
+__device__ __forceinline__ void rank_select_by(const uint64_t* keys, int n, int k, uint64_t* out) {
+  const int i = threadIdx.x / T, s = threadIdx.x % T;
   const uint64_t key = i < n ? keys[i] : 0ull;
+  int c = 0;
+  if constexpr (T == 16) {  // n <= 64
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c += (s + 16 * j < n && keys[s + 16 * j] > key) ? 1 : 0;
+  } else {
+#pragma unroll 4
+    for (int o = s; o < n; o += T) c += keys[o] > key ? 1 : 0;
+  }
+#pragma unroll
+  for (int off = T / 2; off > 0; off >>= 1) c += __shfl_xor_sync(adt::kFullMask, c, off);
+  if (s == 0 && key != 0ull && c < k) out[c] = key;
+}
+
+// The largest power of two of threads per key that covers all n <= kThreads
+// keys at once (64 keys: 4 comparisons a thread, 128: 16, 256: 64).  Not
+// inlined, nor is the bounded selection: the calls with few keys (k = 8) run
+// past one copy of this code instead of three (an expansion call is too short
+// to hide the instruction fetches).
+__device__ __noinline__ void rank_select(const uint64_t* keys, int n, int k, uint64_t* out) {
+  if (n <= kThreads / 8)
+    rank_select_by<8>(keys, n, k, out);
+  else if (n <= kThreads / 4)
+    rank_select_by<4>(keys, n, k, out);
+  else if (n <= kThreads / 2)
+    rank_select_by<2>(keys, n, k, out);
+  else
+    rank_select_by<1>(keys, n, k, out);
+}
+
+// Sixty-four groups of 16 threads hold one value each; the rank of a group's
+// value among them (the groups with a larger one, ties to the lower group
+// when `ties`), in every thread of the group.
+template <bool ties, class T>
+__device__ __noinline__ int rank_of_64(const T* v) {
+  static_assert(kThreads == 64 * 16, "16 threads for each of 64 values");
+  const int g = threadIdx.x >> 4, s = threadIdx.x & 15;
+  const T mine = v[g];
   int c = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int o = s + 16 * j;
-    c += (o < n && keys[o] > key) ? 1 : 0;
+    const T x = v[o];
+    c += (x > mine || (ties && x == mine && o < g)) ? 1 : 0;
   }
 #pragma unroll
   for (int off = 8; off > 0; off >>= 1) c += __shfl_xor_sync(adt::kFullMask, c, off);
-  if (s == 0 && key != 0ull && c < k) out[c] = key;
+  return c;
 }
 
+struct SelectScratch {
+  uint64_t group[64];
+  uint64_t bound;
+  unsigned count;
+};
+
+// out[rank] = key for the k (<= 64) largest of the distinct keys key_at(0..n)
+// (0 entries skipped); out[] zeroed by the caller.  The k-th largest of 64
+// group maxima (key i belongs to group i % 64, so that runs of large keys
+// spread over the groups) bounds the k largest from below; the keys at or
+// above it, about 64 ln(64 / (64 - k)) of n in no particular order, are
+// gathered in list[kCandCap] and ranked against each other.  False, and
+// nothing written, when more than kCandCap keys reach the bound.  Block-wide.
+template <class KeyAt>
+__device__ bool bound_select(KeyAt key_at, int n, int k, SelectScratch* sc, uint64_t* list, uint64_t* out) {
+  const int tid = threadIdx.x;
+  uint64_t mx = 0ull;
+  for (int i = (tid >> 4) + 64 * (tid & 15); i < n; i += kThreads) {
+    const uint64_t key = key_at(i);
+    mx = key > mx ? key : mx;
+  }
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) {
+    const uint64_t o = __shfl_xor_sync(adt::kFullMask, mx, off);
+    mx = o > mx ? o : mx;
+  }
+  if ((tid & 15) == 0) sc->group[tid >> 4] = mx;
+  if (tid == 0) {
+    sc->bound = 0ull;  // kept when fewer than k groups hold a key
+    sc->count = 0u;
+  }
+  __syncthreads();
+  const int rk = rank_of_64<false>(sc->group);
+  if ((tid & 15) == 0 && rk == k - 1 && mx != 0ull) sc->bound = mx;
+  __syncthreads();
+  const uint64_t bound = sc->bound;
+  for (int i = tid; i < n; i += kThreads) {
+    const uint64_t key = key_at(i);
+    if (key >= bound && key != 0ull) {
+      const unsigned pos = atomicAdd(&sc->count, 1u);
+      if (pos < static_cast<unsigned>(kCandCap)) list[pos] = key;
+    }
+  }
+  __syncthreads();
+  const int cnt = static_cast<int>(sc->count);
+  if (cnt > kCandCap) return false;
+  rank_select(list, cnt, k, out);
+  return true;
+}
+
+// The same for n <= kCandCap keys in shared memory: up to kDirectRank of them
+// are ranked as they are (two barriers less).
+constexpr int kDirectRank = 128;
+
+__device__ __noinline__ void select_many(const uint64_t* keys, int n, int k, SelectScratch* sc, uint64_t* list,
+                                         uint64_t* out) {
+  if (n <= kDirectRank)
+    rank_select(keys, n, k, out);
+  else
+    (void)bound_select([&](int i) { return keys[i]; }, n, k, sc, list, out);
+}
+
+__device__ __forceinline__ void select_shared(const uint64_t* keys, int n, int k, SelectScratch* sc, uint64_t* list,
+                                              uint64_t* out) {
+  if (n <= kThreads / 16)
+    rank_select_by<16>(keys, n, k, out);
+  else
+    select_many(keys, n, k, sc, list, out);
+}
+
+// kNarrow: at most 8 children per row, a CTA's share of the row in one tile,
+// and at most 64 cross-row keys or no next frontier (the 7B-shape draft).
+// kPlain: no guidance, temperature 1.
+// The paths it leaves out are only code there, but a call is a chain of short
+// phases and each one fetched past them: with all of them a call at F = 8,
+// V = 65536, k = 8 took 0.4 us longer.
+template <bool kNarrow, bool kPlain>
 __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) {
-  extern __shared__ __align__(16) float vals[];    // [min(per, kTile)] staged logits (x2 with guidance)
+  extern __shared__ __align__(16) float vals[];    // [min(per, tile)] staged logits (x2 with guidance)
   __shared__ uint64_t cand[kCandCap];              // keys at or above the CTA's bound
   __shared__ uint64_t wl[kWarps][kMaxK];           // overflow path: each warp's top k
-  __shared__ float s_bw[kWarps], s_mw[kWarps], s_sw[kWarps];
+  __shared__ float s_mw[kWarps], s_sw[kWarps];
+  __shared__ float s_hw[2 * kWarps];               // half-warp maxima (k > 32)
+  __shared__ SelectScratch sel_s;
   __shared__ float s_B, s_M;
   __shared__ unsigned s_cnt;
   __shared__ uint64_t ctl[kMaxK];                  // this CTA's top k
@@ -270,10 +386,11 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   // This CTA's share of the row: [c0, c1), c0 a multiple of 4.
   const int per = (((p.V + C - 1) / C) + 3) & ~3;
   const int c0 = min(p.V, rank * per), c1 = min(p.V, c0 + per);
-  const int ntiles = (c1 - c0 + kTile - 1) / kTile;
+  const int tile = kNarrow ? per : p.tile;
+  const int ntiles = kNarrow ? 1 : (c1 - c0 + tile - 1) / tile;
   const float* row = p.logits + static_cast<int64_t>(r) * p.ld;
   const float* row_u = p.logits_u ? p.logits_u + static_cast<int64_t>(r) * p.ld : nullptr;
-  float* vals_u = vals + min(per, kTile);  // used only with guidance
+  float* vals_u = vals + min(per, tile);  // used only with guidance
 
   // The row's frontier score and id, read now by the threads that write the
   // children at the end: the loads' latency hides behind the passes.
@@ -283,67 +400,57 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   uint32_t phase = 0;
   bool ok = true;
 
-  // Pass 1: each thread's two largest values (ties kept).  Thread tid takes
-  // elements tid, tid + 1024, ... of every tile.
-  float v1 = -INFINITY, v2 = -INFINITY;
+  // Pass 1: each thread's largest value.  Thread tid takes elements tid,
+  // tid + 1024, ... of every tile.
+  float v1 = -INFINITY;
   for (int tt = 0; tt < ntiles; ++tt) {
-    const int t0 = c0 + tt * kTile, t1 = min(c1, t0 + kTile);
+    const int t0 = c0 + tt * tile, t1 = min(c1, t0 + tile);
     if (tt > 0) __syncthreads();  // the previous tile is consumed
-    ok &= stage_tile(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
+    ok &= stage_tile<kPlain>(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
 #pragma unroll 8
-    for (int i = tid; i < t1 - t0; i += kThreads) {
-      const float x = vals[i];
-      v2 = fmaxf(v2, fminf(v1, x));
-      v1 = fmaxf(v1, x);
-    }
+    for (int i = tid; i < t1 - t0; i += kThreads) v1 = fmaxf(v1, vals[i]);
   }
   if (!ok && tid == 0) adt::raise_error(p.err, ADT_DEVERR_TIMEOUT);
   // The bound B: a value with at least k of the CTA's logits at or above it,
-  // so that its k best are among those >= B.  For k <= 32: the k-th largest
-  // of the 32 warp maxima (ranked by counting in warp 0).  For larger k: per
-  // warp, the largest of its 64 lane values (two per lane) with k of them at
-  // or above it; B is the largest of those.
+  // so that its k best are among those >= B.  For k <= 32 the k-th largest of
+  // the 32 warp maxima (ranked by counting in warp 0), for larger k the k-th
+  // largest of the 64 half-warp maxima (16 threads rank each): about
+  // 32 ln(32 / (32 - k)) or 64 ln(64 / (64 - k)) logits reach it, 60 for
+  // k = 39 of a 2048-logit share.
   {
-    const float mw = adt::warp_max(v1);
-    float bw = -INFINITY;
-    if (K > 32) {
-      int g1 = 0, g2 = 0;
-      for (int j = 0; j < 32; ++j) {
-        const float o1 = __shfl_sync(adt::kFullMask, v1, j), o2 = __shfl_sync(adt::kFullMask, v2, j);
-        g1 += (o1 >= v1) + (o2 >= v1);
-        g2 += (o1 >= v2) + (o2 >= v2);
-      }
-      float cb = -INFINITY;
-      if (g1 >= K) cb = v1;
-      if (g2 >= K) cb = fmaxf(cb, v2);
-      bw = adt::warp_max(cb);
-    }
-    if (lane == 0) {
-      s_bw[warp] = bw;
-      s_mw[warp] = mw;
-    }
+    float hw = v1;
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) hw = fmaxf(hw, __shfl_xor_sync(adt::kFullMask, hw, off));
+    const float mw = fmaxf(hw, __shfl_xor_sync(adt::kFullMask, hw, 16));
+    if (!kNarrow && (lane & 15) == 0) s_hw[tid >> 4] = hw;
+    if (lane == 0) s_mw[warp] = mw;
   }
   __syncthreads();
+  if (!kNarrow && K > 32) {
+    const int rk = rank_of_64<true>(s_hw);
+    if ((tid & 15) == 0 && rk == K - 1) s_B = s_hw[tid >> 4];
+  }
   if (warp == 0) {
     const float mv = s_mw[lane];
     const float mmax = adt::warp_max(mv);
-    const float b = K <= 32 ? warp_kth_largest(mv, K, lane) : adt::warp_max(s_bw[lane]);
+    const float b = kNarrow || K <= 32 ? warp_kth_largest(mv, K, lane) : 0.f;
     if (lane == 0) {
-      s_B = b;
+      if (kNarrow || K <= 32) s_B = b;
       s_M = mmax;
     }
   }
   __syncthreads();
   const float B = s_B, M = s_M;
-  // Pass 2: sum of exp(x - M) as 2^(x log2 e - M log2 e); gather the keys of
-  // values >= B (few: shared-memory atomics, no per-element vote).
+  // Pass 2: sum of exp(x - M) as 2^(x log2 e - Ml), Ml = M log2 e rounded (the
+  // rounding, common to the CTA's terms, is taken out of the sum); gather the
+  // keys of values >= B (few: shared-memory atomics, no per-element vote).
   const float Ml = M == -INFINITY ? 0.f : M * kLog2e;
   float sa[4] = {0.f, 0.f, 0.f, 0.f};
   for (int tt = 0; tt < ntiles; ++tt) {
-    const int t0 = c0 + tt * kTile, t1 = min(c1, t0 + kTile);
+    const int t0 = c0 + tt * tile, t1 = min(c1, t0 + tile);
     if (ntiles > 1) {
       __syncthreads();
-      ok &= stage_tile(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
+      ok &= stage_tile<kPlain>(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
     }
     const int n = t1 - t0;
     for (int i0 = tid; i0 < n; i0 += 4 * kThreads) {
@@ -367,10 +474,8 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   }
   __syncthreads();
   const int cnt = static_cast<int>(s_cnt);
-  if (cnt <= 64) {
-    rank_select64(cand, cnt, K, ctl);
-  } else if (cnt <= kCandCap) {
-    rank_select(cand, cnt, K, ctl);
+  if (cnt <= kCandCap) {
+    select_shared(cand, cnt, K, &sel_s, &wl[0][0], ctl);
   } else {
     // Overflow (very many values at or above B): each warp keeps its k
     // largest by insertion in a third pass, then the lists merge.
@@ -379,10 +484,10 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
     WarpTopK tk;
     uint64_t thr = 0ull;
     for (int tt = 0; tt < ntiles; ++tt) {
-      const int t0 = c0 + tt * kTile, t1 = min(c1, t0 + kTile);
+      const int t0 = c0 + tt * tile, t1 = min(c1, t0 + tile);
       if (ntiles > 1) {
         __syncthreads();
-        ok &= stage_tile(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
+        ok &= stage_tile<kPlain>(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
       }
       const int n = t1 - t0;
       for (int base = warp * 32; base < n; base += kThreads) {
@@ -405,7 +510,8 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
     if (lane < K) dst[lane] = ctl[lane];
     if (lane + 32 < K) dst[lane + 32] = ctl[lane + 32];
     const float S = adt::warp_sum(s_sw[lane]);  // kWarps == 32
-    if (lane == 0) *cl.map_shared_rank(&cl_ms[rank], 0) = make_float2(M, S);
+    const float off = M == -INFINITY ? 0.f : fmaf(M, kLog2e, -Ml);  // exact: every term is 2^off too large
+    if (lane == 0) *cl.map_shared_rank(&cl_ms[rank], 0) = make_float2(M, S * ex2_approx(-off));
   }
   sm100::cluster_arrive_release();
   sm100::cluster_wait_acquire();
@@ -424,10 +530,10 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
     if (lane == 0) s_lse = static_cast<double>(Mr) + static_cast<double>(logf(S));
   }
   __syncthreads();
-  if (C * K <= 64)
-    rank_select64(cl_keys, C * K, K, rowl);
+  if constexpr (kNarrow)
+    rank_select_by<16>(cl_keys, C * K, K, rowl);
   else
-    rank_select(cl_keys, C * K, K, rowl);
+    select_shared(cl_keys, C * K, K, &sel_s, cand, rowl);
   __syncthreads();
   if (writer) {
     const uint64_t key = rowl[tid];
@@ -464,24 +570,33 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
 
   // ---- last row: next frontier across all rows.
   const int nc = p.F * K;
-  if (p.k_keep <= kMaxK && nc <= kCandCap) {
-    for (int i = tid; i < nc; i += kThreads) cross_s[i] = __ldcg(p.cross_keys + i);
+  auto cross_key = [&](int i) { return __ldcg(p.cross_keys + i); };
+  bool done = kNarrow;
+  if (kNarrow || p.k_keep <= kMaxK) {
     for (int i = tid; i < kMaxK; i += kThreads) rowl[i] = 0ull;
+    if constexpr (kNarrow) {
+      if (tid < nc) cross_s[tid] = cross_key(tid);
+      __syncthreads();
+      rank_select_by<16>(cross_s, nc, p.k_keep, rowl);
+    } else if (nc <= kCandCap) {
+      for (int i = tid; i < nc; i += kThreads) cross_s[i] = cross_key(i);
+      __syncthreads();
+      select_shared(cross_s, nc, p.k_keep, &sel_s, &wl[0][0], rowl);
+      done = true;
+    } else {
+      __syncthreads();
+      done = bound_select(cross_key, nc, p.k_keep, &sel_s, cross_s, rowl);
+    }
     __syncthreads();
-    if (nc <= 64)
-      rank_select64(cross_s, nc, p.k_keep, rowl);
-    else
-      rank_select(cross_s, nc, p.k_keep, rowl);
-    __syncthreads();
-    if (tid < p.k_keep) {
+    if (done && tid < p.k_keep) {
       const uint64_t key = rowl[tid];
       const int32_t c = static_cast<int32_t>(adt::select_key_index(key));
       p.keep[tid] = c;
       if (p.nscore) p.nscore[tid] = adt::select_key_value(key);
       if (p.nid) p.nid[tid] = p.id_base + c;
     }
-  } else {
-    auto cross_key = [&](int i) { return __ldcg(p.cross_keys + i); };
+  }
+  if (!kNarrow && !done) {
     const uint64_t thr3 = adt::block_topk_threshold<kThreads>(cross_key, nc, p.k_keep, &rs);
     collect_sorted(cross_key, nc, thr3, p.k_keep, sel, &s_cnt);
     for (int j = tid; j < p.k_keep; j += kThreads) {
@@ -495,10 +610,22 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   if (tid == 0) *p.all_ticket = 0u;
 }
 
-// CTAs per row (the cluster size).
-int expand_cluster(int V) {
-  const int c = (V + kValuesPerCta - 1) / kValuesPerCta;
-  return c < 1 ? 1 : (c > kMaxCluster ? kMaxCluster : c);
+// CTAs per row (the cluster size): one per kValuesPerCta logits, as long as
+// all rows' clusters run at once.  A CTA fills an SM (1024 threads of 63
+// registers) and the GPCs leave a part of the SMs out of a cluster's reach,
+// so the limit is four fifths of the SMs; beyond it the rows take two waves:
+// F = 39, V = 16384, k = 39, without the next frontier: 15.7, 13.2, 11.4, 6.9
+// and 7.6 us with 8, 6, 4, 2 and 1 CTAs per row; F = 20, k = 20: 10.6, 6.1,
+// 6.0, 6.2 and 7.3 us; at V = 65536 14.4, 12.1 and 18.5 us with 4, 2 and 1
+// (F = 39) and 12.0, 7.1, 7.3 and 11.4 with 8, 6, 4 and 2 (F = 20).  Sizes
+// cut down stay even: three CTAs a row cost 9.0 against 7.6 us with two (F =
+// 39, guided).
+int expand_cluster(int F, int V, int sm_count) {
+  int c = (V + kValuesPerCta - 1) / kValuesPerCta;
+  c = c < 1 ? 1 : (c > kMaxCluster ? kMaxCluster : c);
+  const int most = 4 * sm_count / (5 * F);
+  if (c > most) c = most < 2 ? 1 : most / 2 * 2;
+  return c;
 }
 
 // Workspace layout.  The completion counter sits at a fixed offset at the
@@ -812,15 +939,17 @@ static adt_status expand_impl(const float* logits, const float* logits_u, float 
   p.cross_keys = reinterpret_cast<uint64_t*>(ws + w.cross_keys);
   p.all_ticket = reinterpret_cast<unsigned*>(ws + w.all_ticket);
   p.err = info.error_word;
-  const int C = expand_cluster(V);
+  const int C = expand_cluster(F, V, info.sm_count);
   const int per = ((V + C - 1) / C + 3) & ~3;
-  const size_t dyn = static_cast<size_t>(per < kTile ? per : kTile) * sizeof(float) * (logits_u ? 2 : 1);
+  p.tile = logits_u ? kTileGuided : kTile;
+  const size_t dyn = static_cast<size_t>(per < p.tile ? per : p.tile) * sizeof(float) * (logits_u ? 2 : 1);
   static unsigned configured[2] = {0u, 0u};  // bit per device (< 64)
   unsigned& word = configured[(info.device >> 5) & 1];
   const unsigned bit = 1u << (info.device & 31);
   if (!(__atomic_load_n(&word, __ATOMIC_ACQUIRE) & bit)) {
-    ADT_CUDA_TRY(cudaFuncSetAttribute(expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      static_cast<int>(2 * kTile * sizeof(float))));
+    for (auto k : {expand_kernel<true, true>, expand_kernel<true, false>, expand_kernel<false, false>})
+      ADT_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        static_cast<int>(kTile * sizeof(float))));
     __atomic_fetch_or(&word, bit, __ATOMIC_ACQ_REL);
   }
   cudaLaunchConfig_t cfg = {};
@@ -836,7 +965,11 @@ static adt_status expand_impl(const float* logits, const float* logits_u, float 
   attr[1] = adt::pdl_attribute();
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, expand_kernel, p));
+  const bool narrow = k_child <= kThreads / 16 / kMaxCluster && per <= p.tile &&
+                      (!keep_idx || F * k_child <= kThreads / 16);
+  const bool plain = !logits_u && !p.use_T;
+  ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, !narrow ? expand_kernel<false, false>
+                                        : plain ? expand_kernel<true, true> : expand_kernel<true, false>, p));
   return adt::launch_status();
 }
 

@@ -1,0 +1,73 @@
+"""Wide drafts: the expansion's selections past 8 children a row (64 group
+maxima bound the keys that are ranked, radix selection where too many reach
+the bound), and its split of a row over fewer CTAs when there are many rows."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_cases import ensure_built
+from paper_2512_21857_gb300 import synth
+from test_parity_cfg import run_expand_cfg
+from test_parity_expand_rerank import check_expand, run_expand
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    ensure_built()
+
+
+@pytest.mark.parametrize("F,V,k,keep", [
+    (8, 65536, 8, 8), (9, 65536, 8, 8),      # 64 and 72 cross-row keys
+    (8, 65536, 9, 9),                        # 72 keys in a row's lists
+    (3, 16384, 32, 32), (3, 16384, 33, 33),  # warp maxima, half-warp maxima
+    (20, 65536, 20, 20),                     # 6 CTAs a row
+    (39, 65536, 39, 64),                     # 2 CTAs a row, a full tile each, 64 kept of 1521
+    (16, 4100, 64, 64),                      # 1024 cross-row keys
+    (130, 40000, 5, 100),                    # one CTA a row, two tiles; k_keep past 64
+])
+def test_expand_wide_matches_oracle(F, V, k, keep):
+    logits = synth.f32_normal((F, V), F + V + k, "logits", std=3.0)
+    fscore = synth.f32_normal((F,), F + V + k, "fs", std=1.0) - 2.0
+    got, _ = run_expand(logits, fscore, None, k, keep, base=5)
+    check_expand(got, oracle.tree_expand(logits, fscore, k, keep, child_id_base=5), keep)
+
+
+@pytest.mark.parametrize("F,V,k", [(39, 65536, 39), (2, 4098, 8)])
+def test_expand_guided_tiles_match_oracle(F, V, k):
+    """Guidance halves the tile: two CTAs a row stage two tiles each at V = 65536."""
+    V4 = (V + 3) // 4 * 4
+    cond, uncond = (synth.f32_normal((F, V4), V + i, "l", std=3.0) for i in range(2))
+    fscore = synth.f32_normal((F,), V, "fs", std=1.0)
+    got = run_expand_cfg(cond, uncond, fscore, None, k, k)
+    check_expand(got, oracle.tree_expand(oracle.cfg_logits(cond, uncond, 3.0), fscore, k, k), k)
+
+
+def test_expand_cross_row_overflow_takes_the_radix_path():
+    """63 of 64 children of every row far above the last one: the bound of
+    the cross-row selection is a last child, and more keys reach it than the
+    candidate buffer holds."""
+    F, V, k = 40, 2048, 64
+    logits = synth.f32_normal((F, V), 5, "logits", std=0.5)
+    g = np.random.default_rng(5)
+    for r in range(F):
+        logits[r, g.choice(V, size=63, replace=False)] += np.float32(30.0)
+    fscore = synth.f32_normal((F,), 6, "fs", std=0.1)
+    got, _ = run_expand(logits, fscore, None, k, 64)
+    check_expand(got, oracle.tree_expand(logits, fscore, k, 64), 64)
+
+
+@pytest.mark.parametrize("n_top", [129, 1025])
+def test_expand_ties_past_the_direct_ranking(n_top):
+    """n_top copies of the largest value in one CTA's share, k = 40: ranked
+    after a second bound (129), or past the candidate buffer (1025)."""
+    V, F, k = 65536, 2, 40
+    g = np.random.default_rng(n_top)
+    logits = g.normal(0.0, 1.0, size=(F, V)).astype(np.float32)
+    pos = np.sort(g.choice(8192, size=n_top, replace=False)) + 8192 * 3
+    logits[0, pos] = np.float32(7.0)
+    fscore = np.array([-1.0, -0.25], np.float32)
+    got, _ = run_expand(logits, fscore, None, k, k)
+    assert got["child_token"][:k].tolist() == pos[:k].tolist()
+    check_expand(got, oracle.tree_expand(logits, fscore, k, k), k)
