@@ -661,231 +661,224 @@ struct RerankParams {
   int32_t* parents;
   int32_t* cand_index;
   int32_t* depth;
-  int32_t* node_of;       // [C]  workspace
-  int32_t* cand_of_node;  // [n_nodes] workspace
   unsigned* err;
 };
 
-// Shared-memory rerank for up to kRerankSmall candidates and nodes: a
-// candidate is selected when fewer than n_nodes - 1 candidate keys exceed
-// its own (a warp takes a key and its lanes count), node ids follow
-// ascending candidate index (block scan of the selection flags), and the
-// node maps, parents and depths never leave shared memory.  With at most
-// kRerankBound nodes to select from at least 64 candidates, only the keys
-// at or above a bound are ranked: every warp's two largest keys (over a
-// strided view, so that every warp holds candidates) give 64 distinct keys,
-// and the (n_nodes - 1)-th largest of them has at least n_nodes - 1 keys at
-// or above it.
-constexpr int kRerankSmall = 1024;
-constexpr int kRerankBound = 64;
+// Rerank of any pool.  The scores are mapped, order kept, to kRerankBins
+// bins over their range; a histogram gives the bin that holds the
+// (n_nodes - 1)-th best, every candidate of a better bin is selected, and the
+// few of that bin are ranked against each other (when they are too many --
+// nearly all scores equal -- a radix select finds the threshold key instead).
+// Node ids follow ascending candidate index (one scan over the warps'
+// counts of all tiles), and node maps, parents and depths stay in shared
+// memory.  Bound by latency: 3.3 us at C = 328, n = 64 (4.6 us when every
+// warp's two largest keys gave the bound), 3.8 us at C = 858, n = 256 (46.3 us
+// with all keys ranked against each other), 6.1 us at C = 6123, n = 256 and
+// 11.8 us at C = 12207 (9.6 and 16.6 us with radix passes over the keys in
+// memory).  M: scores a thread keeps in registers (C <= 1024 M); 0: they are
+// read again where needed.
+constexpr int kRerankBins = 1024;
+constexpr int kRerankList = 1024;      // candidates of the threshold bin ranked by counting
+constexpr int kRerankMaxC = 65536;
+constexpr int kRerankMaxNodes = 4096;
+constexpr int kRerankMaxTiles = kRerankMaxC / kRerankThreads;
+constexpr int kRerankRegs = 8;
 
-__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
+struct RerankShared {
+  int par[kRerankMaxNodes];              // a node's candidate index, then its parent's node id
+  uint64_t list[kRerankList];
+  int hist[kRerankBins];
+  int tot[kRerankMaxTiles * 32];         // selected per (tile, warp), then their exclusive prefix
+  float fmax[32], fmin[32];
+  int wsum[32];
+  int bin, need, count, nlist, bad;
+  adt::RadixScratch rs;
+};
+
+// Exclusive prefix of one value per thread over the block.
+__device__ __forceinline__ int rerank_block_scan(int v, int* wsum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int incl = v;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t w = __shfl_xor_sync(adt::kFullMask, v, o);
-    v = w > v ? w : v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(adt::kFullMask, incl, o);
+    if (lane >= o) incl += y;
   }
-  return v;
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  const int w = wsum[lane];
+  int wi = w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(adt::kFullMask, wi, o);
+    if (lane >= o) wi += y;
+  }
+  return __shfl_sync(adt::kFullMask, wi - w, warp) + incl - v;
 }
 
-__global__ void __launch_bounds__(kRerankThreads) rerank_small_kernel(const RerankParams p) {
-  __shared__ uint64_t keys[kRerankSmall];
-  __shared__ int node_of[kRerankSmall];
-  __shared__ int cand_of_node[kRerankSmall + 1];
-  __shared__ int par[kRerankSmall + 1];
-  __shared__ int cpar_s[kRerankSmall];
-  __shared__ uint64_t list[kRerankSmall];
-  __shared__ uint64_t s_top[2 * 32];
-  __shared__ uint64_t s_bound;
-  __shared__ int s_nlist;
-  __shared__ int warp_tot[32];
-  __shared__ int s_bad;
+template <int M>
+__global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankParams p) {
+  extern __shared__ uint16_t node_of[];  // [C]: a candidate's node id, 0xFFFF if not selected
+  __shared__ RerankShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int need = p.n_nodes - 1, C = p.C;
+  const int tiles = (C + kRerankThreads - 1) / kRerankThreads;
+  sh.hist[tid] = 0;
+  if (tid == 0) {
+    sh.nlist = 0;
+    sh.bad = 0;
+  }
   adt::pdl_wait_then_release();
   if (tid == 0) {
     p.tokens[0] = *p.root;
     p.parents[0] = -1;
     if (p.cand_index) p.cand_index[0] = -1;
     if (p.depth) p.depth[0] = 0;
-    par[0] = -1;
-    s_bad = 0;
-    s_nlist = 0;
+    sh.par[0] = -1;
   }
   if (need == 0) return;
-  // Candidate tid (C <= kRerankThreads): its key, token and parent id, all
-  // loaded in one round; node_of holds the selection flags until the scan.
-  uint64_t key = 0ull;
-  int tok = 0;
-  if (tid < C) {
-    key = adt::select_key(p.cscore[tid], static_cast<uint32_t>(tid));
-    tok = p.ctok[tid];
-    cpar_s[tid] = p.cpar[tid];
-    keys[tid] = key;
-    node_of[tid] = 0;
+  float x[M ? M : 1];
+  float mx = -INFINITY, mn = INFINITY;
+  auto see = [&](float v) {
+    mx = fmaxf(mx, v);
+    mn = v > -INFINITY ? fminf(mn, v) : mn;
+  };
+  if constexpr (M > 0) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int i = tid + m * kRerankThreads;
+      x[m] = i < C ? p.cscore[i] : -INFINITY;
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) see(x[m]);
+  } else {
+    for (int i = tid; i < C; i += kRerankThreads) see(p.cscore[i]);
   }
-  __syncthreads();
-  if (need <= kRerankBound && C >= 2 * 32) {
-    {
-      const int i = lane * 32 + warp;  // every warp sees at least two candidates
-      const uint64_t v = i < C ? keys[i] : 0ull;
-      const uint64_t m1 = warp_max_u64(v);
-      const uint64_t m2 = warp_max_u64(v == m1 ? 0ull : v);
-      if (lane == 0) {
-        s_top[warp] = m1;
-        s_top[warp + 32] = m2;
+  // f(m, candidate, score) for every candidate of this thread, tile by tile.
+  auto each = [&](auto f) {
+    if constexpr (M > 0) {
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if (m < tiles) f(m, tid + m * kRerankThreads, x[m]);
+    } else {
+      for (int m = 0; m < tiles; ++m) {
+        const int i = tid + m * kRerankThreads;
+        f(m, i, i < C ? p.cscore[i] : -INFINITY);
       }
     }
-    __syncthreads();
-    {
-      // warp w ranks s_top[w] and s_top[w + 32] among the 64
-      const uint64_t x = s_top[lane], y = s_top[lane + 32];
-      const uint64_t a = s_top[warp], c = s_top[warp + 32];
-      const int ra = __popc(__ballot_sync(adt::kFullMask, x > a)) + __popc(__ballot_sync(adt::kFullMask, y > a));
-      const int rc = __popc(__ballot_sync(adt::kFullMask, x > c)) + __popc(__ballot_sync(adt::kFullMask, y > c));
-      if (lane == 0 && ra == need - 1) s_bound = a;
-      if (lane == 0 && rc == need - 1) s_bound = c;
-    }
-    __syncthreads();
-    if (tid < C && key >= s_bound) list[atomicAdd(&s_nlist, 1)] = key;
-    __syncthreads();
-    const int nl = s_nlist;
-    for (int e = warp; e < nl; e += kRerankThreads / 32) {
-      const uint64_t ke = list[e];
-      int rk = 0;
-      for (int j = 0; j < nl; j += 32) rk += __popc(__ballot_sync(adt::kFullMask, j + lane < nl && list[j + lane] > ke));
-      if (lane == 0 && rk < need) node_of[adt::select_key_index(ke)] = 1;
-    }
-  } else {
-    for (int i = warp; i < C; i += kRerankThreads / 32) {
-      const uint64_t ki = keys[i];
-      int rk = 0;
-      for (int j = 0; j < C; j += 32) rk += __popc(__ballot_sync(adt::kFullMask, j + lane < C && keys[j + lane] > ki));
-      if (lane == 0) node_of[i] = rk < need ? 1 : 0;
+  };
+  mx = adt::warp_max(mx);
+  mn = -adt::warp_max(-mn);
+  if (lane == 0) {
+    sh.fmax[warp] = mx;
+    sh.fmin[warp] = mn;
+  }
+  __syncthreads();
+  mx = adt::warp_max(sh.fmax[lane]);
+  mn = -adt::warp_max(-sh.fmin[lane]);
+  // Non-increasing in the score (each operation rounds monotonically), so a
+  // better bin holds better scores only; equal scores (and +0, -0) share one.
+  const float span = mx - mn;
+  const float scale = span > 0.f && span < INFINITY ? (kRerankBins - 1) / span : 0.f;
+  auto bin_of = [&](float v) -> int {
+    return v > -INFINITY ? min(kRerankBins - 1, static_cast<int>((mx - v) * scale)) : kRerankBins - 1;
+  };
+  each([&](int, int i, float v) {
+    if (i < C) atomicAdd(&sh.hist[bin_of(v)], 1);
+  });
+  __syncthreads();
+  {
+    const int h = sh.hist[tid];
+    const int before = rerank_block_scan(h, sh.wsum);
+    if (before < need && need <= before + h) {
+      sh.bin = tid;
+      sh.need = need - before;
+      sh.count = h;
     }
   }
   __syncthreads();
-  const bool sel = tid < C && node_of[tid] != 0;
-  // node id = 1 + selected candidates of lower index (block exclusive scan)
-  const unsigned bal = __ballot_sync(adt::kFullMask, sel);
-  if (lane == 0) warp_tot[warp] = __popc(bal);
-  __syncthreads();
-  int before = __popc(bal & ((1u << lane) - 1u));
-  for (int w = 0; w < warp; ++w) before += warp_tot[w];
-  if (tid < C) {
-    const int node = sel ? 1 + before : -1;
-    node_of[tid] = node;
-    if (sel) {
-      cand_of_node[node] = tid;
-      p.tokens[node] = tok;
-      if (p.cand_index) p.cand_index[node] = tid;
+  const int tbin = sh.bin, tneed = sh.need, tcount = sh.count;
+  // Bit m of `sel`: candidate tid + 1024 m is selected.
+  uint64_t sel = 0ull;
+  if (tcount == tneed) {
+    each([&](int m, int i, float v) {
+      if (i < C && bin_of(v) <= tbin) sel |= 1ull << m;
+    });
+  } else if (tcount <= kRerankList) {
+    each([&](int m, int i, float v) {
+      if (i >= C) return;
+      const int bn = bin_of(v);
+      if (bn < tbin) sel |= 1ull << m;
+      if (bn == tbin) sh.list[atomicAdd(&sh.nlist, 1)] = adt::select_key(v, static_cast<uint32_t>(i));
+    });
+    __syncthreads();
+    // The tneed-th best of the list: warps take keys, lanes count.
+    for (int e = warp; e < tcount; e += kRerankThreads / 32) {
+      const uint64_t ke = sh.list[e];
+      int c = 0;
+      for (int j = lane; j < tcount; j += 32) c += sh.list[j] > ke ? 1 : 0;
+      c = __reduce_add_sync(adt::kFullMask, c);
+      if (lane == 0 && c == tneed - 1) sh.bin = e;  // keys are distinct: one entry has this rank
     }
+    __syncthreads();
+    const uint64_t thr = sh.list[sh.bin];
+    each([&](int m, int i, float v) {
+      if (i < C && bin_of(v) == tbin && adt::select_key(v, static_cast<uint32_t>(i)) >= thr) sel |= 1ull << m;
+    });
+  } else {
+    const uint64_t thr = adt::block_topk_threshold<kRerankThreads>(
+        [&](int i) { return adt::select_key(p.cscore[i], static_cast<uint32_t>(i)); }, C, need, &sh.rs);
+    each([&](int m, int i, float v) {
+      if (i < C && adt::select_key(v, static_cast<uint32_t>(i)) >= thr) sel |= 1ull << m;
+    });
+  }
+  // Node ids in ascending candidate order.
+  for (int m = 0; m < tiles; ++m) {
+    const unsigned bal = __ballot_sync(adt::kFullMask, (sel >> m) & 1ull);
+    if (lane == 0) sh.tot[m * 32 + warp] = __popc(bal);
+  }
+  __syncthreads();
+  {
+    const int nt = tiles * 32;  // <= 2 kRerankThreads
+    const int a = 2 * tid < nt ? sh.tot[2 * tid] : 0, b = 2 * tid + 1 < nt ? sh.tot[2 * tid + 1] : 0;
+    const int before = rerank_block_scan(a + b, sh.wsum);
+    if (2 * tid < nt) sh.tot[2 * tid] = before;
+    if (2 * tid + 1 < nt) sh.tot[2 * tid + 1] = before + a;
+  }
+  __syncthreads();
+  for (int m = 0; m < tiles; ++m) {
+    const int i = tid + m * kRerankThreads;
+    const bool mine = (sel >> m) & 1ull;
+    const unsigned bal = __ballot_sync(adt::kFullMask, mine);
+    const int node = 1 + sh.tot[m * 32 + warp] + __popc(bal & ((1u << lane) - 1u));
+    if (i < C) node_of[i] = mine ? static_cast<uint16_t>(node) : 0xFFFFu;
+    if (mine) sh.par[node] = i;
   }
   __syncthreads();
   for (int node = 1 + tid; node <= need; node += kRerankThreads) {
-    const int pc = cpar_s[cand_of_node[node]];
+    const int c = sh.par[node];
+    const int tok = p.ctok[c], pc = p.cpar[c];
+    p.tokens[node] = tok;
+    if (p.cand_index) p.cand_index[node] = c;
     int pr = 0;
     if (pc >= 0) {
-      pr = pc < C ? node_of[pc] : -1;
-      if (pr < 0 || pr >= node) {
-        s_bad = 1;
+      const int of = pc < C ? node_of[pc] : 0xFFFF;
+      pr = of;
+      if (of == 0xFFFF || of >= node) {
+        sh.bad = 1;
         pr = 0;
       }
     }
-    par[node] = pr;
+    sh.par[node] = pr;
     p.parents[node] = pr;
   }
   __syncthreads();
-  if (s_bad && tid == 0) adt::raise_error(p.err, ADT_DEVERR_BAD_TREE);
+  if (sh.bad && tid == 0) adt::raise_error(p.err, ADT_DEVERR_BAD_TREE);
   if (p.depth) {
     for (int node = 1 + tid; node <= need; node += kRerankThreads) {
       int d = 0, j = node;
       while (j > 0 && d <= need) {
-        j = par[j];
-        ++d;
-      }
-      p.depth[node] = d;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankParams p) {
-  __shared__ adt::RadixScratch rs;
-  __shared__ int warp_tot[32];
-  __shared__ int warp_excl[32];
-  __shared__ int s_running;
-  __shared__ int s_tile;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int need = p.n_nodes - 1;
-  adt::pdl_wait_then_release();
-  if (tid == 0) {
-    p.tokens[0] = *p.root;
-    p.parents[0] = -1;
-    if (p.cand_index) p.cand_index[0] = -1;
-    if (p.depth) p.depth[0] = 0;
-    p.cand_of_node[0] = -1;
-    s_running = 0;
-  }
-  if (need == 0) return;
-  auto key_at = [&](int i) { return adt::select_key(p.cscore[i], static_cast<uint32_t>(i)); };
-  const uint64_t thr = adt::block_topk_threshold<kRerankThreads>(key_at, p.C, need, &rs);
-  // Node ids in ascending candidate order: block-wide exclusive scan of the flags.
-  for (int base = 0; base < p.C; base += kRerankThreads) {
-    const int i = base + tid;
-    const bool f = i < p.C && key_at(i) >= thr;
-    const unsigned bal = __ballot_sync(adt::kFullMask, f);
-    const int in_warp = __popc(bal & ((1u << lane) - 1u));
-    if (lane == 0) warp_tot[warp] = __popc(bal);
-    __syncthreads();
-    if (warp == 0) {
-      const int v = warp_tot[lane];
-      int incl = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(adt::kFullMask, incl, o);
-        if (lane >= o) incl += y;
-      }
-      warp_excl[lane] = incl - v;
-      if (lane == 31) s_tile = incl;
-    }
-    __syncthreads();
-    const int before = s_running + warp_excl[warp] + in_warp;
-    if (i < p.C) {
-      const int node = f ? 1 + before : -1;
-      if (node >= 1 && node <= need) {
-        p.node_of[i] = node;
-        p.tokens[node] = p.ctok[i];
-        p.cand_of_node[node] = i;
-        if (p.cand_index) p.cand_index[node] = i;
-      } else {
-        p.node_of[i] = -1;
-      }
-    }
-    __syncthreads();
-    if (tid == 0) s_running += s_tile;
-    __syncthreads();
-  }
-  __threadfence_block();
-  __syncthreads();
-  for (int node = 1 + tid; node <= need; node += kRerankThreads) {
-    const int c = p.cand_of_node[node];
-    const int pc = p.cpar[c];
-    int par = 0;
-    if (pc >= 0) {
-      par = (pc < p.C) ? p.node_of[pc] : -1;
-      if (par < 0 || par >= node) {
-        adt::raise_error(p.err, ADT_DEVERR_BAD_TREE);
-        par = 0;
-      }
-    }
-    p.parents[node] = par;
-  }
-  __threadfence_block();
-  __syncthreads();
-  if (p.depth) {
-    for (int node = 1 + tid; node <= need; node += kRerankThreads) {
-      int d = 0, j = node;
-      while (j > 0 && d <= need) {
-        j = p.parents[j];
+        j = sh.par[j];
         ++d;
       }
       p.depth[node] = d;
@@ -1020,13 +1013,12 @@ adt_status adt_tree_rerank(const int32_t* cand_token, const float* cand_score,
                            size_t workspace_bytes, void* stream) {
   adt::TraceRange trace_("adt_tree_rerank");
   ADT_REQUIRE(cand_token && cand_score && cand_parent && root_token && tokens && parents);
-  ADT_REQUIRE(C >= 1 && C <= 65536 && n_nodes >= 1 && n_nodes <= C + 1 && n_nodes <= 4096);
+  ADT_REQUIRE(C >= 1 && C <= kRerankMaxC && n_nodes >= 1 && n_nodes <= C + 1 && n_nodes <= kRerankMaxNodes);
   const size_t need = adt_tree_rerank_workspace_size(C);
   if (!workspace || workspace_bytes < need || !adt::aligned16(workspace)) return ADT_ERR_WORKSPACE;
   adt::DeviceInfo info;
   adt_status st = adt::device_info(&info);
   if (st != ADT_OK) return st;
-  uint8_t* ws = static_cast<uint8_t*>(workspace);
   RerankParams p;
   p.ctok = cand_token;
   p.cscore = cand_score;
@@ -1038,8 +1030,6 @@ adt_status adt_tree_rerank(const int32_t* cand_token, const float* cand_score,
   p.parents = parents;
   p.cand_index = cand_index;
   p.depth = depth;
-  p.node_of = reinterpret_cast<int32_t*>(ws);
-  p.cand_of_node = reinterpret_cast<int32_t*>(ws + adt::align_up(static_cast<size_t>(C) * sizeof(int32_t), 256));
   p.err = info.error_word;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(1, 1, 1);
@@ -1048,10 +1038,23 @@ adt_status adt_tree_rerank(const int32_t* cand_token, const float* cand_score,
   cudaLaunchAttribute attr[1] = {adt::pdl_attribute()};
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (C <= kRerankSmall && C <= kRerankThreads && n_nodes <= kRerankSmall + 1)
-    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_small_kernel, p));
+  static unsigned configured[2] = {0u, 0u};  // bit per device (< 64)
+  unsigned& word = configured[(info.device >> 5) & 1];
+  const unsigned bit = 1u << (info.device & 31);
+  if (!(__atomic_load_n(&word, __ATOMIC_ACQUIRE) & bit)) {
+    ADT_CUDA_TRY(cudaFuncSetAttribute(rerank_kernel<kRerankRegs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kRerankRegs * kRerankThreads * static_cast<int>(sizeof(uint16_t))));
+    ADT_CUDA_TRY(cudaFuncSetAttribute(rerank_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kRerankMaxC * static_cast<int>(sizeof(uint16_t))));
+    __atomic_fetch_or(&word, bit, __ATOMIC_ACQ_REL);
+  }
+  cfg.dynamicSmemBytes = static_cast<size_t>(C) * sizeof(uint16_t);
+  if (C <= kRerankThreads)
+    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<1>, p));
+  else if (C <= kRerankRegs * kRerankThreads)
+    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<kRerankRegs>, p));
   else
-    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel, p));
+    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<0>, p));
   return adt::launch_status();
 }
 

@@ -1,14 +1,17 @@
 """Wide drafts: the expansion's selections past 8 children a row (64 group
 maxima bound the keys that are ranked, radix selection where too many reach
-the bound), and its split of a row over fewer CTAs when there are many rows."""
+the bound), its split of a row over fewer CTAs when there are many rows, and
+the rerank of large pools (score bins, then the threshold bin ranked)."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
-from gpu_cases import ensure_built
+from gpu_cases import ensure_built, f32, i32
+from paper_2512_21857_gb300 import binding as B
 from paper_2512_21857_gb300 import synth
 from test_parity_cfg import run_expand_cfg
-from test_parity_expand_rerank import check_expand, run_expand
+from test_parity_expand_rerank import _random_pool, check_expand, run_expand
 
 pytestmark = pytest.mark.gpu
 
@@ -71,3 +74,32 @@ def test_expand_ties_past_the_direct_ranking(n_top):
     got, _ = run_expand(logits, fscore, None, k, k)
     assert got["child_token"][:k].tolist() == pos[:k].tolist()
     check_expand(got, oracle.tree_expand(logits, fscore, k, k), k)
+
+
+def _rerank(tok, sc, par, n):
+    C = len(tok)
+    res = {x: torch.empty(n, dtype=torch.int32, device="cuda") for x in ("tokens", "parents", "cand_index", "depth")}
+    ws = B.zeroed_workspace(B.adt_tree_rerank_workspace_size(C))
+    B.adt_tree_rerank(i32(tok), f32(sc), i32(par), C, i32([7]), n, workspace=ws, **res)
+    torch.cuda.synchronize()
+    return {x: t.cpu().numpy() for x, t in res.items()}
+
+
+@pytest.mark.parametrize("C,n", [(328, 64), (1024, 256), (1025, 2), (6123, 256), (8192, 4096), (8193, 257),
+                                 (40000, 64), (65536, 4096)])
+@pytest.mark.parametrize("scores", ["grown", "flat", "outlier", "masked"])
+def test_rerank_large_pools(C, n, scores):
+    """Scores as grown; all equal; all but one far away in one bin; the last third -inf."""
+    tok, sc, par = _random_pool(C, seed=C + n)
+    if scores == "flat":
+        sc = np.full_like(sc, -3.0)
+    elif scores == "outlier":
+        sc = sc.copy()
+        sc[0] = np.float32(1e30)
+        par[:] = -1
+    elif scores == "masked":
+        sc, par = sc.copy(), np.full_like(par, -1)
+        sc[2 * C // 3:] = -np.inf
+    got, ref = _rerank(tok, sc, par, n), oracle.tree_rerank(tok, sc, par, 7, n)
+    for key in got:
+        assert np.array_equal(got[key], ref[key]), key
