@@ -120,6 +120,8 @@ struct TcParams {
   int B, H, Hkv, group, max_kv, splits;
   int qtiles;         // 64-row query tiles per tree: ceil(max_nodes / 64)
   int cluster_merge;
+  int max_tree;       // largest tree accepted: 64 * qtiles
+  int heads, row_stride;  // 128-row kernel: heads per CTA and rows per head
   float scale_log2;
   __nv_bfloat16* out;
   float* lse;
@@ -296,6 +298,44 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
   return false;
 }
 
+// The tree of a launch slot.  With several trees (up to 32) the launch slots
+// go to the trees by decreasing prefix length (ties: lower index): the CTAs
+// are dispatched in slot order, so the longest streams start first and the
+// short ones fill in behind them instead of a late long tree ending the
+// launch.  Every warp ranks the trees itself (one lane per tree), from the
+// same single round of loads the one-tree path makes.
+struct TreeSlot {
+  int b, node0, n, total_nodes, L;
+};
+
+__device__ __forceinline__ TreeSlot tree_of_slot(const TcParams& p, int slot, int lane) {
+  TreeSlot t;
+  if (p.B > 1 && p.B <= 32) {
+    const bool mine = lane < p.B;
+    const int kl = mine ? p.kv_len[lane] : 0;
+    const int off = mine ? p.offs[lane] : 0;
+    t.total_nodes = p.offs[p.B];
+    int rank = 0;
+    for (int i = 0; i < p.B; ++i) {
+      const int o = __shfl_sync(adt::kFullMask, kl, i);
+      rank += (o > kl || (o == kl && i < lane)) ? 1 : 0;
+    }
+    const unsigned hit = __ballot_sync(adt::kFullMask, mine && rank == slot);
+    t.b = hit ? __ffs(hit) - 1 : slot;
+    t.L = __shfl_sync(adt::kFullMask, kl, t.b);
+    t.node0 = __shfl_sync(adt::kFullMask, off, t.b);
+    const int next = __shfl_sync(adt::kFullMask, off, (t.b + 1) & 31);
+    t.n = (t.b + 1 < p.B ? next : t.total_nodes) - t.node0;
+  } else {
+    t.b = slot;
+    t.node0 = p.offs[t.b];
+    t.n = p.offs[t.b + 1] - t.node0;
+    t.total_nodes = p.offs[p.B];
+    t.L = p.kv_len[t.b];
+  }
+  return t;
+}
+
 // kLarge: trees of more than 64 nodes (query tiles, one mask word per tree
 // unit); otherwise one tile and one word, kept in registers.
 
@@ -366,36 +406,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the previous kernel in the stream has completed (immediate when this
   // launch does not overlap one).
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
-  // The tree of this CTA.  With several trees (up to 32) the launch slots
-  // go to the trees by decreasing prefix length (ties: lower index): the
-  // CTAs are dispatched in slot order, so the longest streams start first
-  // and the short ones fill in behind them instead of a late long tree
-  // ending the launch.  Every warp ranks the trees itself (one lane per
-  // tree), from the same single round of loads the one-tree path makes.
-  int b, node0, n, total_nodes, L;
-  if (p.B > 1 && p.B <= 32) {
-    const bool mine = lane < p.B;
-    const int kl = mine ? p.kv_len[lane] : 0;
-    const int off = mine ? p.offs[lane] : 0;
-    total_nodes = p.offs[p.B];
-    int rank = 0;
-    for (int i = 0; i < p.B; ++i) {
-      const int o = __shfl_sync(adt::kFullMask, kl, i);
-      rank += (o > kl || (o == kl && i < lane)) ? 1 : 0;
-    }
-    const unsigned hit = __ballot_sync(adt::kFullMask, mine && rank == slot);
-    b = hit ? __ffs(hit) - 1 : slot;
-    L = __shfl_sync(adt::kFullMask, kl, b);
-    node0 = __shfl_sync(adt::kFullMask, off, b);
-    const int next = __shfl_sync(adt::kFullMask, off, (b + 1) & 31);
-    n = (b + 1 < p.B ? next : total_nodes) - node0;
-  } else {
-    b = slot;
-    node0 = p.offs[b];
-    n = p.offs[b + 1] - node0;
-    total_nodes = p.offs[p.B];
-    L = p.kv_len[b];
-  }
+  const TreeSlot ts = tree_of_slot(p, slot, lane);
+  const int b = ts.b, node0 = ts.node0, n = ts.n, total_nodes = ts.total_nodes, L = ts.L;
 
   // Conditions that hold for every CTA of this (tree, head, tile): all
   // leave here, handing back the tensor memory.  A tile past the end of its
@@ -1180,6 +1192,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) p.tickets[bh] = 0u;
 }
 
+#include "tree_attn_wide.cuh"
+
 // ---------------------------------------------------------------- host side
 
 // Splits per (tree, head): about one CTA per SM, at most one split per chunk
@@ -1240,10 +1254,10 @@ void load_encode() {
 }
 
 // 4-D map of a cache (d, pos, kv head, tree) with the 128-byte swizzle and
-// boxes of 64 columns x 128 positions; positions at or past max_kv read as
-// zero.
+// boxes of 64 columns x box_keys positions; positions at or past max_kv read
+// as zero.
 adt_status make_cache_map(CUtensorMap* map, const void* base, int D, int max_kv, int Hkv, int B, int64_t sh,
-                          int64_t sb) {
+                          int64_t sb, int box_keys = kChunk) {
   std::call_once(g_encode_once, load_encode);
   if (!g_encode) return ADT_ERR_CUDA;
   const int64_t span = static_cast<int64_t>(max_kv > 0 ? max_kv : 1);
@@ -1251,7 +1265,7 @@ adt_status make_cache_map(CUtensorMap* map, const void* base, int D, int max_kv,
                         static_cast<cuuint64_t>(B)};
   cuuint64_t strides[3] = {static_cast<cuuint64_t>(D) * 2, static_cast<cuuint64_t>(sh > 0 ? sh : span * D) * 2,
                            static_cast<cuuint64_t>(sb > 0 ? sb : span * D * Hkv) * 2};
-  cuuint32_t box[4] = {64, kChunk, 1, 1};
+  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(box_keys), 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1309,6 +1323,33 @@ int max_active_clusters(int D, bool large, int cluster, int dev) {
   return num;
 }
 
+template <int D>
+int wide_active_clusters(int cluster, int dev) {
+  static int cache[64][kMaxClusterSplits + 1];  // 0 = not queried yet
+  int& slot = cache[dev & 63][cluster];
+  const int v = __atomic_load_n(&slot, __ATOMIC_ACQUIRE);
+  if (v) return v - 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(cluster), 1, 1);
+  cfg.blockDim = dim3(kWideThreads, 1, 1);
+  cfg.dynamicSmemBytes = WideCfg<D>::kDynSmem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int num = 0;
+  cudaFuncSetAttribute(tree_attn_wide_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, WideCfg<D>::kDynSmem);
+  if (cudaOccupancyMaxActiveClusters(&num, tree_attn_wide_kernel<D>, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    num = 0;
+  }
+  __atomic_store_n(&slot, num + 1, __ATOMIC_RELEASE);
+  return num;
+}
+
 template <int D, bool kLarge>
 adt_status launch(TcParams prm, const void* k_cache, const void* v_cache, int64_t sb, int64_t sh, cudaStream_t st,
                   int dev, bool overlap_previous) {
@@ -1350,9 +1391,85 @@ adt_status launch(TcParams prm, const void* k_cache, const void* v_cache, int64_
   return adt::launch_status();
 }
 
-// Trees of more than 64 nodes take the query-tiled instantiation.
+// CTAs per (tree, head group) of the 128-row kernel: `tiles` tiles with as many
+// key splits as fit the SMs and a portable cluster, all clusters co-resident;
+// 1 where even one split a tile takes more CTAs than there are SMs (the tiles
+// are then CTAs of their own, and those a smaller tree lacks end at once --
+// within a cluster they would hold their SM until its last CTA ends).
+template <int D>
+int wide_cluster(int sm_count, int groups, int tiles, int max_kv, int dev) {
+  const int chunks = (max_kv + kChunk - 1) / kChunk + tiles;
+  int s = sm_count / (groups * tiles);
+  if (s > chunks) s = chunks;
+  if (s > kMaxClusterSplits / tiles) s = kMaxClusterSplits / tiles;
+  while (s > 0 && wide_active_clusters<D>(s * tiles, dev) < groups) --s;
+  return s > 0 ? s * tiles : 1;
+}
+
+// Which calls take the 128-row kernel: heads per CTA (0: the 64-row kernel).
+// A chunk of 128 keys costs it 0.9 us for 128 rows, against 1.1 to 1.2 us for
+// 64, but its fixed cost is 1 to 2 us higher (twice the rows to merge, one
+// thread per row): it pays from about kWideChunks chunks per CTA of the 64-row
+// kernel on.  64-row / 128-row kernel, us: two chunks (H = 8 / 2, D = 64, four
+// trees over 600 keys) 8.8 / 9.6, three (20 / 5 heads, D = 64, 2400 keys)
+// 10.6 / 11.1, nine (32 / 8, D = 128, 4000 keys) 15.3 / 13.2, 20 (256 nodes,
+// 32 heads, D = 128, 2400 keys) 29.9 / 19.1.
+constexpr int kWideChunks = 6;
+
+int wide_heads(const TcParams& prm, int sm_count) {
+  const int heads = prm.qtiles > 1 ? 1 : prm.group % 2 == 0 ? 2 : 0;
+  const int chunks = (prm.max_kv + kChunk - 1) / kChunk + (prm.qtiles + 1) / 2;
+  const int ctas = prm.B * prm.qtiles * prm.H * prm.splits;
+  const int waves = (ctas + sm_count - 1) / sm_count;
+  // (More splits than a cluster holds merge in fp32 through the workspace.)
+  return prm.splits <= kMaxClusterSplits && chunks * waves >= kWideChunks * prm.splits ? heads : 0;
+}
+
+template <int D>
+adt_status launch_wide(TcParams prm, int heads, const void* k_cache, const void* v_cache, int64_t sb, int64_t sh,
+                       cudaStream_t st, int dev, int sm_count, bool overlap_previous) {
+  static unsigned configured[2] = {0u, 0u};  // bit per device (< 64)
+  const unsigned bit = 1u << (dev & 31);
+  unsigned& word = configured[dev >> 5];
+  if (!(__atomic_load_n(&word, __ATOMIC_ACQUIRE) & bit)) {
+    ADT_CUDA_TRY(cudaFuncSetAttribute(tree_attn_wide_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      WideCfg<D>::kDynSmem));
+    __atomic_fetch_or(&word, bit, __ATOMIC_ACQ_REL);
+  }
+  CUtensorMap tm_k, tm_v;
+  adt_status s1 = make_cache_map(&tm_k, k_cache, D, prm.max_kv, prm.Hkv, prm.B, sh, sb);
+  if (s1 != ADT_OK) return s1;
+  s1 = make_cache_map(&tm_v, v_cache, D, prm.max_kv, prm.Hkv, prm.B, sh, sb);
+  if (s1 != ADT_OK) return s1;
+  prm.heads = heads;
+  prm.row_stride = kWideRows / heads;
+  const int tiles = (prm.max_tree + kWideRows - 1) / kWideRows;
+  const int groups = prm.B * (prm.H / heads);
+  const int cluster = wide_cluster<D>(sm_count, groups, tiles, prm.max_kv, dev);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(prm.H / heads),
+                     static_cast<unsigned>(cluster > 1 ? prm.B : prm.B * tiles));
+  cfg.blockDim = dim3(kWideThreads, 1, 1);
+  cfg.dynamicSmemBytes = WideCfg<D>::kDynSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1] = adt::pdl_attribute();
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap_previous ? 2 : 1;
+  ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, tree_attn_wide_kernel<D>, tm_k, tm_v, prm));
+  return adt::launch_status();
+}
+
 adt_status launch_any(const TcParams& prm, int D, const void* k_cache, const void* v_cache, int64_t sb, int64_t sh,
-                      cudaStream_t st, int dev, bool overlap_previous) {
+                      cudaStream_t st, int dev, int sm_count, bool overlap_previous) {
+  const int heads = wide_heads(prm, sm_count);
+  if (heads)
+    return D == 128 ? launch_wide<128>(prm, heads, k_cache, v_cache, sb, sh, st, dev, sm_count, overlap_previous)
+                    : launch_wide<64>(prm, heads, k_cache, v_cache, sb, sh, st, dev, sm_count, overlap_previous);
   const bool large = prm.qtiles > 1;
   if (D == 128)
     return large ? launch<128, true>(prm, k_cache, v_cache, sb, sh, st, dev, overlap_previous)
@@ -1403,6 +1520,7 @@ TcParams make_params(const adt_bf16* q, const int32_t* kv_len, const adt_bf16* k
   prm.max_kv = max_kv;
   prm.splits = splits;
   prm.qtiles = qtiles_for(max_nodes);
+  prm.max_tree = kMaxNodes * prm.qtiles;
   prm.scale_log2 = scale * kLog2e;
   prm.out = reinterpret_cast<__nv_bfloat16*>(out);
   prm.lse = lse;
@@ -1455,7 +1573,7 @@ adt_status adt_tree_attn(const adt_bf16* q, const adt_bf16* k_cache, const adt_b
   prm.part_ml = reinterpret_cast<float2*>(ws + w.part_ml);
   prm.tickets = reinterpret_cast<unsigned*>(ws + w.tickets);
   cudaStream_t s = adt::as_stream(stream);
-  return launch_any(prm, D, k_cache, v_cache, cache_stride_b, cache_stride_h, s, info.device, true);
+  return launch_any(prm, D, k_cache, v_cache, cache_stride_b, cache_stride_h, s, info.device, info.sm_count, true);
 }
 
 }  // extern "C"
@@ -1565,6 +1683,6 @@ extern "C" adt_status adt_tree_attn_noalloc(const adt_bf16* q, const adt_bf16* k
   prm.part_o = reinterpret_cast<float*>(ws + w.part_o);
   prm.part_ml = reinterpret_cast<float2*>(ws + w.part_ml);
   prm.tickets = reinterpret_cast<unsigned*>(ws + w.tickets);
-  return launch_any(prm, D, k_cache, v_cache, cache_stride_b, cache_stride_h, s, info.device, false);
+  return launch_any(prm, D, k_cache, v_cache, cache_stride_b, cache_stride_h, s, info.device, info.sm_count, false);
 }
 
