@@ -38,6 +38,10 @@
 // at D = 128 a row travels as O / l in fp16 with a power-of-two scale (half
 // the bytes of fp32, which the copies between SMs are bound by).  With more
 // splits they merge through the workspace.
+//
+// Launches with long key ranges per CTA whose tiles can hold more than 64 rows
+// (trees of more than 64 nodes, grouped query heads) take the 128-row kernel
+// of tree_attn_wide.cuh instead (see wide_heads).
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_fp16.h>
