@@ -111,18 +111,33 @@ def _check(status: int, where: str) -> None:
         raise AdtError(status, where)
 
 
+# A call's marshalling is on a decode loop's critical path (the launch itself
+# takes 2 us): addresses go to ctypes as plain integers, and the current
+# stream's handle is read without building a torch.cuda.Stream for it (3.0 ->
+# 0.2 us a call).
+
 def _ptr(t):
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError("expected a CUDA tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and _get_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_get_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
+
+
+def _nbytes(t):
+    return t.numel() * t.element_size()
 
 
 def _expect(t, dtype, name):
@@ -182,22 +197,27 @@ def adt_tree_attn(q, k_cache, v_cache, kv_len, k_tree, v_tree, parents, node_off
                   max_nodes, max_kv, softmax_scale, out, lse=None, workspace, cache_stride_b=None,
                   cache_stride_h=None, stream=None) -> None:
     """q, k_tree, v_tree, out: bf16 [Ntot, *, D]; caches bf16 with (b, g, pos, d) strides."""
-    for t, n in ((q, "q"), (k_tree, "k_tree"), (v_tree, "v_tree"), (out, "out")):
-        _expect(t, torch.bfloat16, n)
-    for t, n in ((kv_len, "kv_len"), (parents, "parents"), (node_offsets, "node_offsets")):
-        _expect(t, torch.int32, n)
-    if k_cache.dtype != torch.bfloat16 or v_cache.dtype != torch.bfloat16:
+    bf16, i32 = torch.bfloat16, torch.int32
+    _expect(q, bf16, "q")
+    _expect(k_tree, bf16, "k_tree")
+    _expect(v_tree, bf16, "v_tree")
+    _expect(out, bf16, "out")
+    _expect(kv_len, i32, "kv_len")
+    _expect(parents, i32, "parents")
+    _expect(node_offsets, i32, "node_offsets")
+    if k_cache.dtype != bf16 or v_cache.dtype != bf16:
         raise TypeError("caches must be bf16")
-    if k_cache.stride() != v_cache.stride():
+    strides = k_cache.stride()
+    if strides != v_cache.stride():
         raise ValueError("k_cache and v_cache must share strides")
-    sb = k_cache.stride(0) if cache_stride_b is None else cache_stride_b
-    sh = k_cache.stride(1) if cache_stride_h is None else cache_stride_h
+    sb = strides[0] if cache_stride_b is None else cache_stride_b
+    sh = strides[1] if cache_stride_h is None else cache_stride_h
     if lse is not None:
         _expect(lse, torch.float32, "lse")
     st = lib().adt_tree_attn(_ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(kv_len), sb, sh, _ptr(k_tree),
                              _ptr(v_tree), _ptr(parents), _ptr(node_offsets), B, H, Hkv, D, max_nodes, max_kv,
                              float(softmax_scale), _ptr(out), _ptr(lse), _ptr(workspace),
-                             workspace.numel() * workspace.element_size(), _stream(stream))
+                             _nbytes(workspace), _stream(stream))
     _check(st, "adt_tree_attn")
 
 
@@ -213,7 +233,7 @@ def adt_tree_expand(logits, frontier_score, frontier_id, *, F, V, k_child, k_kee
     st = lib().adt_tree_expand(_ptr(logits), ld, _ptr(frontier_score), _ptr(frontier_id), F, V, k_child, k_keep,
                                float(temperature), int(child_id_base), _ptr(child_token), _ptr(child_logp),
                                _ptr(child_score), _ptr(child_parent), _ptr(keep_idx), _ptr(next_score),
-                               _ptr(next_id), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                               _ptr(next_id), _ptr(workspace), _nbytes(workspace),
                                _stream(stream))
     _check(st, "adt_tree_expand")
 
@@ -232,7 +252,7 @@ def adt_tree_expand_cfg(logits_cond, logits_uncond, frontier_score, frontier_id,
                                    _ptr(frontier_score), _ptr(frontier_id), F, V, k_child, k_keep,
                                    float(temperature), int(child_id_base), _ptr(child_token), _ptr(child_logp),
                                    _ptr(child_score), _ptr(child_parent), _ptr(keep_idx), _ptr(next_score),
-                                   _ptr(next_id), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                   _ptr(next_id), _ptr(workspace), _nbytes(workspace),
                                    _stream(stream))
     _check(st, "adt_tree_expand_cfg")
 
@@ -241,7 +261,7 @@ def adt_tree_rerank(cand_token, cand_score, cand_parent, C, root_token, n_nodes,
                     cand_index=None, depth=None, workspace, stream=None) -> None:
     st = lib().adt_tree_rerank(_ptr(cand_token), _ptr(cand_score), _ptr(cand_parent), int(C), _ptr(root_token),
                                int(n_nodes), _ptr(tokens), _ptr(parents), _ptr(cand_index), _ptr(depth),
-                               _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream))
+                               _ptr(workspace), _nbytes(workspace), _stream(stream))
     _check(st, "adt_tree_rerank")
 
 
@@ -255,7 +275,7 @@ def adt_tree_accept(target_logits, draft_logits, tokens, parents, node_offsets, 
                                _ptr(parents), _ptr(node_offsets), B, V, max_nodes, _ptr(u_accept),
                                _ptr(u_sample), int(mode), float(temperature), _ptr(path), int(max_path),
                                _ptr(accept_len), _ptr(bonus_token), _ptr(ws),
-                               0 if ws is None else ws.numel() * ws.element_size(), _stream(stream))
+                               0 if ws is None else _nbytes(ws), _stream(stream))
     _check(st, "adt_tree_accept")
 
 
