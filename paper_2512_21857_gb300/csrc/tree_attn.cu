@@ -39,6 +39,16 @@
 // the bytes of fp32, which the copies between SMs are bound by).  With more
 // splits they merge through the workspace.
 //
+// Back-to-back launches at the 7B shape (four splits, 41.4 MB, 6.1 us at the
+// measured HBM rate) take 12.6 us, at the LlamaGen shape (six splits, from L2)
+// 7.3 us: the chain from the dependency wait through the first loads to the
+// merge, whose instructions come cold for each launch.  So one copy of the
+// softmax serves every chunk, masks are bit tests on one word per row, the
+// merge is unrolled for the split count's range, and paths off the common one
+// lie behind it (12.9 and 7.4 us with two softmax copies, 64-bit masks and an
+// eight-way merge inline).  One split writes its rows directly (eight ragged
+// trees, 41.9 -> 39.0 us a layer).
+//
 // Launches with long key ranges per CTA whose tiles can hold more than 64 rows
 // (trees of more than 64 nodes, grouped query heads) take the 128-row kernel
 // of tree_attn_wide.cuh instead (see wide_heads).
@@ -47,6 +57,7 @@
 #include <cuda_fp16.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "adt_common.cuh"
 #include "sm100.cuh"
@@ -215,36 +226,42 @@ __device__ __forceinline__ void tmem_st_16x256b_x1(uint32_t taddr, const uint32_
                : "memory");
 }
 
-// x masked to -inf where the keep bit is 0, without branching (a NaN score
-// at a masked position also becomes -inf).
-__device__ __forceinline__ float mask_or_neg_inf(float x, uint32_t keep_bit) {
-  const uint32_t keep = 0u - keep_bit;
-  return __uint_as_float((__float_as_uint(x) & keep) | (0xFF800000u & ~keep));
+// The keep bits of the 32 columns a thread holds of a row (columns 8b + 2t + e
+// of every 8-column block b < 16, t = lane % 4; bit 2b + e): of a tree chunk,
+// from the ancestor words of its two units, and of a prefix chunk that ends
+// after kl keys.
+__device__ __forceinline__ uint32_t unit_bits(uint64_t w, int t4) {
+  uint64_t x = (w >> (2 * t4)) & 0x0303030303030303ull;
+  x = (x | (x >> 6)) & 0x000F000F000F000Full;
+  x = (x | (x >> 12)) & 0x000000FF000000FFull;
+  return static_cast<uint32_t>(x | (x >> 24)) & 0xFFFFu;
+}
+__device__ __forceinline__ uint32_t prefix_bits(int kl, int t4) {
+  uint32_t bits = 0u;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int nb = min(max((kl - 2 * t4 - e + 7) >> 3, 0), 16);  // blocks whose column e is in the prefix
+    bits |= (nb == 16 ? 0x55555555u : 0x55555555u & ((1u << (2 * nb)) - 1u)) << e;
+  }
+  return bits;
 }
 
-// Softmax of one chunk for the two rows (a, b) a thread holds: NB 8-column
-// blocks (8 for 64 keys, 16 for 128), scores in sa / sb (raw Q.K), keep
-// masks (bit c = column c) applied only when `masked`.  Updates the lazily
-// raised maxima mu (log2 units), returns the rescale factors of O (and of
-// the row sums, which the tensor core accumulates from the same bf16
-// probabilities) and the probabilities packed in column pairs.
-template <int NB>
-__device__ __forceinline__ void chunk_softmax(float (&sa)[32], float (&sb)[32], bool masked, uint64_t ka0,
-                                              uint64_t ka1, uint64_t kb0, uint64_t kb1, int t4, float scale,
-                                              float& mu_a, float& mu_b, float& alpha_a,
-                                              float& alpha_b, uint32_t (&pa)[16], uint32_t (&pb)[16]) {
+// Softmax of one chunk for the two rows (a, b) a thread holds: scores in sa /
+// sb (raw Q.K), keep bits applied only when `masked` (a chunk of one 64-key
+// unit is one whose upper half is masked: one copy of this code is fetched
+// instead of two).  Updates the lazily raised maxima mu (log2 units), returns
+// the rescale factors of O (and of the row sums, which the tensor core
+// accumulates from the same bf16 probabilities) and the probabilities packed
+// in column pairs.
+__device__ __forceinline__ void chunk_softmax(float (&sa)[32], float (&sb)[32], bool masked, uint32_t ka, uint32_t kb,
+                                              float scale, float& mu_a, float& mu_b, float& alpha_a, float& alpha_b,
+                                              uint32_t (&pa)[16], uint32_t (&pb)[16]) {
+  constexpr int NB = 16;
   if (masked) {
-    const int sh = 2 * t4;
-    const uint64_t a0 = ka0 >> sh, a1 = ka1 >> sh, b0 = kb0 >> sh, b1 = kb1 >> sh;
 #pragma unroll
-    for (int bk = 0; bk < NB; ++bk) {
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int c = 8 * (bk & 7) + e;
-        const uint64_t ma = bk < 8 ? a0 : a1, mb = bk < 8 ? b0 : b1;
-        sa[2 * bk + e] = mask_or_neg_inf(sa[2 * bk + e], static_cast<uint32_t>(ma >> c) & 1u);
-        sb[2 * bk + e] = mask_or_neg_inf(sb[2 * bk + e], static_cast<uint32_t>(mb >> c) & 1u);
-      }
+    for (int i = 0; i < 2 * NB; ++i) {  // a NaN score at a masked position also becomes -inf
+      sa[i] = ka & (1u << i) ? sa[i] : -INFINITY;
+      sb[i] = kb & (1u << i) ? sb[i] : -INFINITY;
     }
   }
   float mxa = sa[0], mxb = sb[0];
@@ -748,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int keys = chunk_keys(j);
       uint32_t r0[32], r1[32];
       tmem_ld_16x256b_x8(tmem + lane_base + sb * kSCols, r0);
-      if (keys == kChunk) tmem_ld_16x256b_x8(tmem + lane_base + sb * kSCols + 64, r1);
+      tmem_ld_16x256b_x8(tmem + lane_base + sb * kSCols + 64, r1);  // a one-unit chunk: stale, masked below
       sm100::tmem_wait_ld();
       // S is in registers: hand the tensor-memory tile back to the MMA warp.
       sm100::tc_fence_before();
@@ -760,23 +777,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       // holds the end of the prefix need a mask.
       const bool tree_j = j < n_tc;
       const int kl = tree_j ? keys : L - chunk_key0(j);
-      const bool masked = tree_j || kl < keys;
-      uint64_t ka0 = ~0ull, ka1 = ~0ull, kb0 = ~0ull, kb1 = ~0ull;
+      const bool masked = tree_j || kl < kChunk;
+      uint32_t ka = ~0u, kb = ~0u;
       if (tree_j) {
         if constexpr (kLarge) {
           // units 2u and 2u + 1 of the tree (rows past the tile have no bits)
           const int u = 2 * (tc0 + j);
-          ka0 = anc[ra][u];
-          kb0 = anc[rb][u];
-          ka1 = u + 1 < kUnits ? anc[ra][u + 1] : 0ull;
-          kb1 = u + 1 < kUnits ? anc[rb][u + 1] : 0ull;
+          ka = unit_bits(anc[ra][u], t4);
+          kb = unit_bits(anc[rb][u], t4);
+          if (keys == kChunk) {
+            ka |= unit_bits(anc[ra][u + 1], t4) << 16;
+            kb |= unit_bits(anc[rb][u + 1], t4) << 16;
+          }
         } else {
-          ka0 = ama;
-          kb0 = amb;
+          ka = unit_bits(ama, t4);
+          kb = unit_bits(amb, t4);
         }
-      } else if (kl < keys) {
-        ka0 = kb0 = kl >= 64 ? ~0ull : ((1ull << kl) - 1ull);
-        ka1 = kb1 = kl >= 128 ? ~0ull : (kl > 64 ? ((1ull << (kl - 64)) - 1ull) : 0ull);
+      } else if (kl < kChunk) {
+        ka = kb = prefix_bits(kl, t4);
       }
       float sa[32], sbv[32];
 #pragma unroll
@@ -792,10 +810,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       uint32_t pa[16], pb[16];
       float alpha_a, alpha_b;
-      if (keys == kChunk)
-        chunk_softmax<16>(sa, sbv, masked, ka0, ka1, kb0, kb1, t4, scale, mua, mub, alpha_a, alpha_b, pa, pb);
-      else
-        chunk_softmax<8>(sa, sbv, masked, ka0, ka1, kb0, kb1, t4, scale, mua, mub, alpha_a, alpha_b, pa, pb);
+      chunk_softmax(sa, sbv, masked, ka, kb, scale, mua, mub, alpha_a, alpha_b, pa, pb);
 
       // P buffer sb was last read by the PV product of chunk j - 2.
       if (j >= 2 && !__all_sync(adt::kFullMask,
@@ -901,7 +916,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int ra = warp * 16 + g8, rb = ra + 8;
   const int64_t bh = static_cast<int64_t>(blockIdx.z) * p.H + h;  // (tree, tile, head)
   constexpr int kC4 = D / 4;
-  if (p.cluster_merge) {
+  if (p.cluster_merge && S > 1) {
     // Row r of the (tree, head, tile) is merged by split r / rows_per, its owner.
     // Each split writes its partial rows (O unnormalised, then m and l) into
     // its own stage ring, idle now, in row order; one thread sends every
@@ -1004,104 +1019,108 @@ __global__ void __launch_bounds__(kThreads, 1)
       // Thread (row i, 8-column group c8) combines the S normalised partials
       // of that row: weights 2^(m_c - M) l_c / sum (times 2^e_c, the scale the
       // partial was stored at).  A split without keys sent m = -inf (weight 0).
+      // (Unrolled for the split count's range: the code of splits that are not
+      // there would be fetched all the same.)
       constexpr int kC8 = D / 8;
-      for (int idx = tid; idx < rows_mine * kC8; idx += kThreads) {
-        const int i = idx / kC8, c8 = idx % kC8;
-        float2 ml[kMaxClusterSplits];
-        int ec[kMaxClusterSplits];
-        uint4 v[kMaxClusterSplits];
-  #pragma unroll
-        for (int c = 0; c < kMaxClusterSplits; ++c) {
-          if (c < S) {
-            const float* row = slots + (c * rows_per + i) * RS;
-            ml[c] = *reinterpret_cast<const float2*>(row + D / 2);
-            ec[c] = reinterpret_cast<const int*>(row)[D / 2 + 2];
-            v[c] = *reinterpret_cast<const uint4*>(row + c8 * 4);
-          }
-        }
-        float M = -INFINITY;
-  #pragma unroll
-        for (int c = 0; c < kMaxClusterSplits; ++c)
-          if (c < S) M = fmaxf(M, ml[c].x);
-        float lt = 0.f;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  #pragma unroll
-        for (int c = 0; c < kMaxClusterSplits; ++c) {
-          if (c < S) {
-            const float w = ml[c].x == -INFINITY ? 0.f : ex2_approx(ml[c].x - M) * ml[c].y;
-            lt += w;
-            const float ws = w * __uint_as_float(static_cast<uint32_t>(127 + ec[c]) << 23);  // w * 2^e_c
-            const __half2* hv = reinterpret_cast<const __half2*>(&v[c]);
-  #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 f = __half22float2(hv[e]);
-              acc[2 * e] += ws * f.x;
-              acc[2 * e + 1] += ws * f.y;
+      auto merge = [&](auto range) {
+        constexpr int kMost = decltype(range)::value;
+        for (int idx = tid; idx < rows_mine * kC8; idx += kThreads) {
+          const int i = idx / kC8, c8 = idx % kC8;
+          float2 ml[kMost];
+          int ec[kMost];
+          uint4 v[kMost];
+#pragma unroll
+          for (int c = 0; c < kMost; ++c) {
+            if (c < S) {
+              const float* row = slots + (c * rows_per + i) * RS;
+              ml[c] = *reinterpret_cast<const float2*>(row + D / 2);
+              ec[c] = reinterpret_cast<const int*>(row)[D / 2 + 2];
+              v[c] = *reinterpret_cast<const uint4*>(row + c8 * 4);
             }
           }
+          float M = -INFINITY;
+#pragma unroll
+          for (int c = 0; c < kMost; ++c)
+            if (c < S) M = fmaxf(M, ml[c].x);
+          float lt = 0.f;
+          float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int c = 0; c < kMost; ++c) {
+            if (c < S) {
+              const float w = ml[c].x == -INFINITY ? 0.f : ex2_approx(ml[c].x - M) * ml[c].y;
+              lt += w;
+              const float ws = w * __uint_as_float(static_cast<uint32_t>(127 + ec[c]) << 23);  // w * 2^e_c
+              const __half2* hv = reinterpret_cast<const __half2*>(&v[c]);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float2 f = __half22float2(hv[e]);
+                acc[2 * e] += ws * f.x;
+                acc[2 * e + 1] += ws * f.y;
+              }
+            }
+          }
+          const float inv = __fdividef(1.f, lt);
+          __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h) * D + c8 * 8;
+          uint4 pk;
+          pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+          pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+          pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv);
+          pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+          *reinterpret_cast<uint4*>(dst) = pk;
+          if (c8 == 0 && p.lse) p.lse[static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h] = (M + __log2f(lt)) * kLn2;
         }
-        const float inv = __fdividef(1.f, lt);
-        __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h) * D + c8 * 8;
-        uint4 pk;
-        pk.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
-        pk.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-        pk.z = pack_bf16x2(acc[4] * inv, acc[5] * inv);
-        pk.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
-        *reinterpret_cast<uint4*>(dst) = pk;
-        if (c8 == 0 && p.lse) p.lse[static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h] = (M + __log2f(lt)) * kLn2;
-      }
+      };
+      if (S <= 4)
+        merge(std::integral_constant<int, 4>());
+      else
+        merge(std::integral_constant<int, kMaxClusterSplits>());
     } else {
       // Thread (row i, column group c4) combines the S partials of that row:
-      // weights 2^(m_c - M) l_c / sum.  A thread takes two items per pass and
-      // loads every split's values of both before combining either.
-      // A split without keys sent zeros with m = -inf (weight 0).
-      auto merge_item = [&](int idx, float2 (&ml)[kMaxClusterSplits], float4 (&v)[kMaxClusterSplits]) {
-        const int i = idx / kC4, c4 = idx % kC4;
-        float M = ml[0].x;
-  #pragma unroll
-        for (int c = 1; c < kMaxClusterSplits; ++c) M = fmaxf(M, ml[c].x);
-        float lt = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  #pragma unroll
-        for (int c = 0; c < kMaxClusterSplits; ++c) {
-          const float w = ml[c].x == -INFINITY ? 0.f : ex2_approx(ml[c].x - M);
-          lt += w * ml[c].y;
-          acc.x += w * v[c].x;
-          acc.y += w * v[c].y;
-          acc.z += w * v[c].z;
-          acc.w += w * v[c].w;
-        }
-        const float inv = __fdividef(1.f, lt);
-        __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h) * D + c4 * 4;
-        uint2 pk;
-        pk.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-        pk.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-        *reinterpret_cast<uint2*>(dst) = pk;
-        if (c4 == 0 && p.lse) p.lse[static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h] = (M + __log2f(lt)) * kLn2;
-      };
-      auto load_item = [&](int idx, float2 (&ml)[kMaxClusterSplits], float4 (&v)[kMaxClusterSplits]) {
-        const int i = idx / kC4, c4 = idx % kC4;
-  #pragma unroll
-        for (int c = 0; c < kMaxClusterSplits; ++c) {
-          if (c < S) {
-            const float* row = slots + (c * rows_per + i) * RS;
-            ml[c] = *reinterpret_cast<const float2*>(row + D);
-            v[c] = *reinterpret_cast<const float4*>(row + c4 * 4);
-          } else {
-            ml[c] = make_float2(-INFINITY, 0.f);
-            v[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+      // weights 2^(m_c - M) l_c / sum.  A split without keys sent zeros with m
+      // = -inf (weight 0).
+      auto merge = [&](auto range) {
+        constexpr int kMost = decltype(range)::value;
+        for (int idx = tid; idx < rows_mine * kC4; idx += kThreads) {
+          const int i = idx / kC4, c4 = idx % kC4;
+          float2 ml[kMost];
+          float4 v[kMost];
+#pragma unroll
+          for (int c = 0; c < kMost; ++c) {
+            if (c < S) {
+              const float* row = slots + (c * rows_per + i) * RS;
+              ml[c] = *reinterpret_cast<const float2*>(row + D);
+              v[c] = *reinterpret_cast<const float4*>(row + c4 * 4);
+            }
           }
+          float M = -INFINITY;
+#pragma unroll
+          for (int c = 0; c < kMost; ++c)
+            if (c < S) M = fmaxf(M, ml[c].x);
+          float lt = 0.f;
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int c = 0; c < kMost; ++c) {
+            if (c >= S) continue;
+            const float w = ml[c].x == -INFINITY ? 0.f : ex2_approx(ml[c].x - M);
+            lt += w * ml[c].y;
+            acc.x += w * v[c].x;
+            acc.y += w * v[c].y;
+            acc.z += w * v[c].z;
+            acc.w += w * v[c].w;
+          }
+          const float inv = __fdividef(1.f, lt);
+          __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h) * D + c4 * 4;
+          uint2 pk;
+          pk.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+          pk.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+          *reinterpret_cast<uint2*>(dst) = pk;
+          if (c4 == 0 && p.lse) p.lse[static_cast<int64_t>(node0 + row0 + r_lo + i) * p.H + h] = (M + __log2f(lt)) * kLn2;
         }
       };
-      for (int idx = tid; idx < rows_mine * kC4; idx += 2 * kThreads) {
-        float2 ml0[kMaxClusterSplits], ml1[kMaxClusterSplits];
-        float4 v0[kMaxClusterSplits], v1[kMaxClusterSplits];
-        const bool two = idx + kThreads < rows_mine * kC4;
-        load_item(idx, ml0, v0);
-        if (two) load_item(idx + kThreads, ml1, v1);
-        merge_item(idx, ml0, v0);
-        if (two) merge_item(idx + kThreads, ml1, v1);
-      }
+      if (S <= 4)
+        merge(std::integral_constant<int, 4>());
+      else
+        merge(std::integral_constant<int, kMaxClusterSplits>());
     }
     // Every owner has its rows: this CTA's outgoing copies are complete.
     sm100::cluster_wait_acquire();
@@ -1110,6 +1129,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     return;
   }
 
+  if (p.cluster_merge) {
+    // One split: the rows are final.  Normalised, they go through the idle
+    // ring (rows of 16 bytes more than D, so that neither side's accesses
+    // conflict) to be written out 16 bytes at a time.
+    constexpr int kPitch = D * 2 + 16;
+    if (warp < kSoftmaxWarps && have_o) {
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        const int r = half ? rb : ra;
+        const float l = half ? l_rb : l_ra;
+        const float inv = __fdividef(1.f, l);
+        uint8_t* dst = sStage + r * kPitch + t4 * 4;
+#pragma unroll
+        for (int c = 0; c < kOB; ++c)
+#pragma unroll
+          for (int bk = 0; bk < 8; ++bk)
+            *reinterpret_cast<uint32_t*>(dst + c * 128 + bk * 16) =
+                pack_bf16x2(__uint_as_float(o[c][4 * bk + 2 * half]) * inv,
+                            __uint_as_float(o[c][4 * bk + 2 * half + 1]) * inv);
+        if (t4 == 0 && r < nq && p.lse)
+          p.lse[static_cast<int64_t>(node0 + row0 + r) * p.H + h] = ((half ? m_rb : m_ra) + __log2f(l)) * kLn2;
+      }
+      __syncwarp();  // a warp writes out its own 16 rows
+      constexpr int kC8 = D / 8;
+      for (int i = lane; i < 16 * kC8; i += 32) {
+        const int r = warp * 16 + i / kC8, c8 = i % kC8;
+        if (r < nq)
+          *reinterpret_cast<uint4*>(p.out + (static_cast<int64_t>(node0 + row0 + r) * p.H + h) * D + c8 * 8) =
+              *reinterpret_cast<const uint4*>(sStage + r * kPitch + c8 * 16);
+      }
+    }
+    __syncthreads();
+    sm100::tc_fence_after();
+    if (warp == 0) sm100::tmem_dealloc(tmem, kTmemCols);
+    return;
+  }
   // More splits than a portable cluster holds: partials go to the workspace
   // and the CTA that finishes a (tree, head) last merges them.
   float* po = p.part_o + (bh * S + split) * kMaxNodes * D;
