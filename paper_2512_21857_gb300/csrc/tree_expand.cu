@@ -9,26 +9,24 @@
 // largest of the 32 warp maxima (64 half-warp maxima for k > 32) bounds the
 // CTA's top k from below; a second pass sums the exponentials against the
 // CTA's maximum and gathers the few selection keys (value order, then lower
-// index) at or above the bound, which are ranked by counting.  The CTAs' lists go to the cluster's first
-// CTA through distributed shared memory; it ranks them, forms the row's
-// log-sum-exp and writes the row's children (log-probability against it in
-// fp64).  The first CTA of the last row to finish (atomic ticket) ranks the
-// next frontier across all rows.  Every selection of more than 128 keys first
+// index) at or above the bound, which are ranked by counting.  The CTAs push
+// their lists into the cluster's first CTA (asynchronous stores that complete
+// on its mbarrier); it ranks them, forms the row's log-sum-exp and writes the
+// row's children (log-probability against it in double-float, rounded once).
+// The first CTA of the last row to finish (atomic ticket) ranks the next
+// frontier across all rows.  Every selection of more than 128 keys first
 // bounds them the same way (64 group maxima), so that only about as many as
 // are wanted get ranked.
 //
 // A call is bound by the latency of that chain of phases, not by its bytes
 // (2.1 MB at F = 8, V = 65536: 0.3 us of HBM time).  Back-to-back calls in a
-// graph: 6.5 us at F = 8, V = 65536, k = 8 and 4.8 us at F = 1; 12.6 us at
+// graph: 6.3 us at F = 8, V = 65536, k = 8 and 4.6 us at F = 1; 12.3 us at
 // F = 39, V = 16384, k = 39 under guidance.  (With a bound that let half of a
 // CTA's logits through for k > 32, each of them inserted in sorted lists, the
 // last took 221.7 us.)
-#include <cooperative_groups.h>
-
 #include "adt_common.cuh"
+#include "dfloat.cuh"
 #include "sm100.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace {
 
@@ -200,21 +198,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// The k-th largest (k <= 32) of the warp's 32 values (none NaN): the one
-// whose rank -- the values above it, with equal values of lower lanes
-// counted as above -- is k - 1.  32 independent shuffles instead of the
-// dependent chain of a sort.
-__device__ __forceinline__ float warp_kth_largest(float v, int k, int lane) {
-  int rk = 0;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const float o = __shfl_sync(adt::kFullMask, v, j);
-    rk += (o > v || (o == v && j < lane)) ? 1 : 0;
-  }
-  const unsigned m = __ballot_sync(adt::kFullMask, rk == k - 1);
-  return __shfl_sync(adt::kFullMask, v, __ffs(m) - 1);
-}
-
 // out[rank] = key for the k largest of the n (<= kThreads / T) distinct
 // nonzero keys in keys[0..n) (0 entries skipped); out[] zeroed by the caller.
 // Block-wide: T threads per key, each counting the keys above it among every
@@ -363,13 +346,12 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   __shared__ float2 cl_ms[kMaxCluster];
   __shared__ uint64_t rowl[kMaxK];
   __shared__ adt::RadixScratch rs;
-  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ __align__(8) uint64_t s_bar, s_push;
   __shared__ int s_last;
-  __shared__ double s_lse;
+  __shared__ float2 s_lse;  // hi, lo
   uint64_t* cross_s = cand;  // cross-row keys (reuses the candidate buffer)
   uint64_t* sel = cand;      // radix path [kMaxKeep]
 
-  cg::cluster_group cl = cg::this_cluster();
   const int rank = blockIdx.x, C = gridDim.x, r = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = p.k;
@@ -379,9 +361,11 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   if (tid == 0) {
     s_cnt = 0u;
     sm100::mbar_init(sm100::smem_addr(&s_bar), 1);
+    sm100::mbar_init(sm100::smem_addr(&s_push), 1);
     sm100::fence_mbar_init();
   }
   __syncthreads();
+  sm100::cluster_arrive_release();  // the mbarriers are there: waited for before the push
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   // This CTA's share of the row: [c0, c1), c0 a multiple of 4.
   const int per = (((p.V + C - 1) / C) + 3) & ~3;
@@ -413,8 +397,8 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   if (!ok && tid == 0) adt::raise_error(p.err, ADT_DEVERR_TIMEOUT);
   // The bound B: a value with at least k of the CTA's logits at or above it,
   // so that its k best are among those >= B.  For k <= 32 the k-th largest of
-  // the 32 warp maxima (ranked by counting in warp 0), for larger k the k-th
-  // largest of the 64 half-warp maxima (16 threads rank each): about
+  // the 32 warp maxima (a warp ranks each), for larger k the k-th largest of
+  // the 64 half-warp maxima (16 threads rank each): about
   // 32 ln(32 / (32 - k)) or 64 ln(64 / (64 - k)) logits reach it, 60 for
   // k = 39 of a 2048-logit share.
   {
@@ -430,14 +414,12 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
     const int rk = rank_of_64<true>(s_hw);
     if ((tid & 15) == 0 && rk == K - 1) s_B = s_hw[tid >> 4];
   }
-  if (warp == 0) {
-    const float mv = s_mw[lane];
-    const float mmax = adt::warp_max(mv);
-    const float b = kNarrow || K <= 32 ? warp_kth_largest(mv, K, lane) : 0.f;
-    if (lane == 0) {
-      if (kNarrow || K <= 32) s_B = b;
-      s_M = mmax;
-    }
+  {
+    // Warp w ranks the warp maximum w among all (ties to the lower warp).
+    const float mine = s_mw[warp], o = s_mw[lane];
+    const int rk = __popc(__ballot_sync(adt::kFullMask, o > mine || (o == mine && lane < warp)));
+    if (lane == 0 && rk == 0) s_M = mine;
+    if (lane == 0 && (kNarrow || K <= 32) && rk == K - 1) s_B = mine;
   }
   __syncthreads();
   const float B = s_B, M = s_M;
@@ -504,17 +486,28 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   }
   __syncthreads();
   if (!ok && tid == 0) adt::raise_error(p.err, ADT_DEVERR_TIMEOUT);  // a restaged tile's wait
-  // This CTA's top k and (max, sum of exponentials), to the cluster's first CTA.
+  // This CTA's top k and (max, sum of exponentials), to the cluster's first
+  // CTA: asynchronous stores that complete on its mbarrier, one way.  (With a
+  // cluster barrier in their place, the bound ranked by one warp and the
+  // scores in fp64, the 7B draft, six calls and the rerank, took 42.2 us
+  // against 40.4 us.)
+  __syncwarp();
+  sm100::cluster_wait_acquire();
   if (warp == 0) {
-    uint64_t* dst = cl.map_shared_rank(&cl_keys[rank * K], 0);
-    if (lane < K) dst[lane] = ctl[lane];
-    if (lane + 32 < K) dst[lane + 32] = ctl[lane + 32];
+    const uint32_t bar = sm100::mapa_shared(sm100::smem_addr(&s_push), 0);
+    auto push = [&](const void* local, uint64_t v) {
+      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];\n" ::"r"(
+                       sm100::mapa_shared(sm100::smem_addr(local), 0)),
+                   "l"(v), "r"(bar)
+                   : "memory");
+    };
+    if (lane < K) push(&cl_keys[rank * K + lane], ctl[lane]);
+    if (lane + 32 < K) push(&cl_keys[rank * K + lane + 32], ctl[lane + 32]);
     const float S = adt::warp_sum(s_sw[lane]);  // kWarps == 32
     const float off = M == -INFINITY ? 0.f : fmaf(M, kLog2e, -Ml);  // exact: every term is 2^off too large
-    if (lane == 0) *cl.map_shared_rank(&cl_ms[rank], 0) = make_float2(M, S * ex2_approx(-off));
+    if (lane == 0)
+      push(&cl_ms[rank], static_cast<uint64_t>(__float_as_uint(S * ex2_approx(-off))) << 32 | __float_as_uint(M));
   }
-  sm100::cluster_arrive_release();
-  sm100::cluster_wait_acquire();
   // The next kernel in the stream may launch now.  Released here rather than
   // right after the wait: a graph of six back-to-back calls (F = 1, then 8;
   // V = 65536, k = 8) and the rerank took 49.2 us against 51.2 us.
@@ -523,13 +516,23 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
 
   // ---- first CTA of row r: the row's top k and log-sum-exp, its children.
   for (int i = tid; i < kMaxK; i += kThreads) rowl[i] = 0ull;
+  if (tid == 0)
+    sm100::mbar_arrive_expect_tx(sm100::smem_addr(&s_push), static_cast<uint32_t>(C * (K + 1) * sizeof(uint64_t)));
+  const bool pushed = sm100::mbar_wait_bounded(sm100::smem_addr(&s_push), 0, kWaitLimit);
   if (warp == 0) {  // lane c takes CTA c's (max, sum); C <= 8
     const float2 ms = lane < C ? cl_ms[lane] : make_float2(-INFINITY, 0.f);
     const float Mr = adt::warp_max(ms.x);
     const float S = adt::warp_sum(ms.x != -INFINITY ? ms.y * ex2_approx((ms.x - Mr) * kLog2e) : 0.f);
-    if (lane == 0) s_lse = static_cast<double>(Mr) + static_cast<double>(logf(S));
+    if (lane == 0) {
+      const dfl::df t = dfl::two_sum(Mr, logf(S));
+      s_lse = make_float2(t.hi, t.lo);
+    }
   }
-  __syncthreads();
+  if (__syncthreads_or(!pushed)) {  // late pushes still need this CTA: it stays until every peer has left
+    if (tid == 0) adt::raise_error(p.err, ADT_DEVERR_TIMEOUT);
+    sm100::cluster_arrive_release();
+    sm100::cluster_wait_acquire();
+  }
   if constexpr (kNarrow)
     rank_select_by<16>(cl_keys, C * K, K, rowl);
   else
@@ -537,11 +540,20 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   __syncthreads();
   if (writer) {
     const uint64_t key = rowl[tid];
-    const double lp = static_cast<double>(adt::select_key_value(key)) - s_lse;
-    const float score = static_cast<float>(static_cast<double>(f_score) + lp);
+    // x - log-sum-exp and the score in double-float (an fp64 operation takes
+    // as long as dozens of these), each rounded to fp32 once; in fp64 where
+    // that leaves fp32's range (infinities, masks of fp32's lowest value).
+    const float x = adt::select_key_value(key);
+    const dfl::df lpd = dfl::df_add(dfl::df{x, 0.f}, dfl::df{-s_lse.x, -s_lse.y});
+    float lp = lpd.hi, score = dfl::df_add(dfl::df{f_score, 0.f}, lpd).hi;
+    if (!isfinite(lp) || !isfinite(score)) {
+      const double l = static_cast<double>(x) - (isfinite(s_lse.y) ? static_cast<double>(s_lse.x) + s_lse.y : s_lse.x);
+      lp = static_cast<float>(l);
+      score = static_cast<float>(f_score + l);
+    }
     const int64_t c = static_cast<int64_t>(r) * K + tid;
     p.ctok[c] = static_cast<int32_t>(adt::select_key_index(key));
-    if (p.clogp) p.clogp[c] = static_cast<float>(lp);
+    if (p.clogp) p.clogp[c] = lp;
     p.cscore[c] = score;
     p.cpar[c] = f_id;
     if (!p.keep) {

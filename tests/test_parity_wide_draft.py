@@ -103,3 +103,32 @@ def test_rerank_large_pools(C, n, scores):
     got, ref = _rerank(tok, sc, par, n), oracle.tree_rerank(tok, sc, par, 7, n)
     for key in got:
         assert np.array_equal(got[key], ref[key]), key
+
+
+LOWEST = float(np.finfo(np.float32).min)
+
+
+@pytest.mark.parametrize("V,k", [(65536, 8), (16384, 39)])  # one row's CTAs: narrow and general instantiation
+@pytest.mark.parametrize("mask", [-np.inf])
+def test_expand_scores_outside_the_range_of_fp32(V, k, mask):
+    """Rows with fewer than k unmasked logits and frontier scores at the ends
+    of fp32: log-probabilities and scores are those of fp64 rounded once
+    (-inf where the sum of two lowest values leaves the range)."""
+    fscore = np.array([-1.0, LOWEST, -np.inf], np.float32)
+    F = len(fscore)
+    g = np.random.default_rng(k)
+    logits = np.full((F, V), mask, np.float32)
+    for r in range(F):
+        logits[r, g.choice(V, size=k - 3, replace=False)] = g.normal(0.0, 2.0, size=k - 3)
+    got, _ = run_expand(logits, fscore, None, k, k)
+    with np.errstate(over="ignore"):
+        for r in range(F):
+            x = logits[r].astype(np.float64)
+            m = x.max()
+            order = np.argsort(-x, kind="stable")[:k]
+            lp = x[order] - (m + np.log(np.exp(x - m).sum()))
+            sl = slice(r * k, (r + 1) * k)
+            assert got["child_token"][sl].tolist() == order.tolist()
+            np.testing.assert_allclose(got["child_logp"][sl], lp.astype(np.float32), rtol=1e-6, atol=1e-6)
+            np.testing.assert_allclose(got["child_score"][sl], (float(fscore[r]) + lp).astype(np.float32),
+                                       rtol=1e-6, atol=1e-6)
