@@ -522,7 +522,10 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   if (warp == 0) {  // lane c takes CTA c's (max, sum); C <= 8
     const float2 ms = lane < C ? cl_ms[lane] : make_float2(-INFINITY, 0.f);
     const float Mr = adt::warp_max(ms.x);
-    const float S = adt::warp_sum(ms.x != -INFINITY ? ms.y * ex2_approx((ms.x - Mr) * kLog2e) : 0.f);
+    // A weight of 0 drops a share whatever its sum is: one masked with fp32's
+    // lowest value (M log2 e leaves the range) has an infinite one.
+    const float w = ex2_approx((ms.x - Mr) * kLog2e);
+    const float S = adt::warp_sum(ms.x == -INFINITY || w == 0.f ? 0.f : ms.y * w);
     if (lane == 0) {
       const dfl::df t = dfl::two_sum(Mr, logf(S));
       s_lse = make_float2(t.hi, t.lo);

@@ -109,7 +109,7 @@ LOWEST = float(np.finfo(np.float32).min)
 
 
 @pytest.mark.parametrize("V,k", [(65536, 8), (16384, 39)])  # one row's CTAs: narrow and general instantiation
-@pytest.mark.parametrize("mask", [-np.inf])
+@pytest.mark.parametrize("mask", [LOWEST, -np.inf])
 def test_expand_scores_outside_the_range_of_fp32(V, k, mask):
     """Rows with fewer than k unmasked logits and frontier scores at the ends
     of fp32: log-probabilities and scores are those of fp64 rounded once
