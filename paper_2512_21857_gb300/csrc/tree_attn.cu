@@ -40,14 +40,23 @@
 // splits they merge through the workspace.
 //
 // Back-to-back launches at the 7B shape (four splits, 41.4 MB, 6.1 us at the
-// measured HBM rate) take 12.6 us, at the LlamaGen shape (six splits, from L2)
-// 7.3 us: the chain from the dependency wait through the first loads to the
+// measured HBM rate) take 12.5 us, at the LlamaGen shape (six splits, from L2)
+// 7.1 us: the chain from the dependency wait through the first loads to the
 // merge, whose instructions come cold for each launch.  So one copy of the
 // softmax serves every chunk, masks are bit tests on one word per row, the
 // merge is unrolled for the split count's range, and paths off the common one
 // lie behind it (12.9 and 7.4 us with two softmax copies, 64-bit masks and an
-// eight-way merge inline).  One split writes its rows directly (eight ragged
-// trees, 41.9 -> 39.0 us a layer).
+// eight-way merge inline); the first S product waits for the tensor copies
+// alone, and four threads send the merge's rows (7.3 us without).  One split
+// writes its rows directly (eight ragged trees, 41.9 -> 38.4 us a layer).
+//
+// Where the 7B launch's 11 us from the dependency wait to the end go (cycles
+// at 1.93 GHz): 1500 to the first load, 4000 to the first K tile (every CTA's
+// first 128 KB at once), 8800 for the stream (6.3 TB/s), then 1700 for the last
+// softmax, 1800 for its PV product, 1000 to write the partial rows, 1900 to
+// move them, 800 to merge.  Requests ahead of the ring (L2 prefetches of the
+// next chunks, or of the first ones before the dependency wait) made it slower
+// or no faster (12.5-13.5 us): they delay the tiles that are needed first.
 //
 // Launches with long key ranges per CTA whose tiles can hold more than 64 rows
 // (trees of more than 64 nodes, grouped query heads) take the 128-row kernel
@@ -669,8 +678,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == kSMmaWarp) {
     // ------------------------------------------------------------ S = Q K^T
     if (lane == 0) {
-      bool ok = wait_bar(&bars.q_full, 0, &s_abort, p.err, p.wait_limit) &&
-                (!q_tma || wait_bar(&bars.q_tma, 0, &s_abort, p.err, p.wait_limit));
+      // (Q's copies by the softmax warps end in q_full; a tensor copy needs
+      // nothing of theirs, so the first product goes ahead of the masks.)
+      bool ok = wait_bar(q_tma ? &bars.q_tma : &bars.q_full, 0, &s_abort, p.err, p.wait_limit);
       const uint32_t q_addr = sm100::smem_addr(sQ);
       for (int j = 0; ok && j < nch; ++j) {
         const int st = j % NS, sb = j & 1;
@@ -708,8 +718,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         sm100::tc_fence_after();
         const uint32_t v_addr = sm100::smem_addr(sStage + (i % NS) * C::kStageBytes + C::kStageTile);
         const uint32_t pb = p_addr + (i & 1) * C::kPBytes;
-        const int ksteps = chunk_keys(i) / 16;
-        for (int kk = 0; kk < ksteps; ++kk) {
+        const bool whole = chunk_keys(i) == kChunk;
+        // Unrolled: one thread issues the products, and a loop's address
+        // arithmetic is a serial chain between them (the 16 of a chunk took
+        // 985 cycles to issue).
+#pragma unroll
+        for (int kk = 0; kk < kChunk / 16; ++kk) {
+          if (kk == kUnit / 16 && !whole) break;
           const uint64_t da = sm100::smem_desc_sw128(pb + (kk >> 2) * C::kBlock64 + (kk & 3) * 32, 16, 1024);
           const uint64_t db = sm100::smem_desc_sw128(v_addr + kk * 2048, C::kBlock128, 1024);  // LBO: d blocks
           sm100::mma_bf16_ss(tmem + kOCol, da, db, C::kIdescO, (i > 0 || kk > 0) ? 1u : 0u);
@@ -908,6 +923,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       // nothing: weight 0.
       m_ra = m_rb = -INFINITY;
       l_ra = l_rb = 0.f;
+#pragma unroll
+      for (int c = 0; c < kOB; ++c)
+#pragma unroll
+        for (int e = 0; e < 32; ++e) o[c][e] = 0u;
     }
   }
   sm100::tc_fence_before();
@@ -941,14 +960,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int half = 0; half < 2; ++half) {
           const int r = half ? rb : ra;
           const float l = half ? l_rb : l_ra;
-          const float inv = have_o && l > 0.f ? __fdividef(1.f, l) : 0.f;
+          const float inv = l > 0.f ? __fdividef(1.f, l) : 0.f;
           float amax = 0.f;
 #pragma unroll
           for (int c = 0; c < kOB; ++c)
 #pragma unroll
             for (int bk = 0; bk < 8; ++bk)
-              if (have_o)
-                amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(o[c][4 * bk + 2 * half])),
+              amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(o[c][4 * bk + 2 * half])),
                                          fabsf(__uint_as_float(o[c][4 * bk + 2 * half + 1]))));
           amax = fmaxf(amax, __shfl_xor_sync(adt::kFullMask, amax, 1));
           amax = fmaxf(amax, __shfl_xor_sync(adt::kFullMask, amax, 2));
@@ -960,7 +978,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             float* dst = rows_out + r * RS;
             if (t4 == 0) {
               *reinterpret_cast<float2*>(dst + D / 2) =
-                  make_float2(have_o ? (half ? m_rb : m_ra) : -INFINITY, have_o ? l : 0.f);
+                  make_float2(half ? m_rb : m_ra, l);
               reinterpret_cast<int*>(dst)[D / 2 + 2] = e;
             }
 #pragma unroll
@@ -968,9 +986,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
               for (int bk = 0; bk < 8; ++bk)
                 reinterpret_cast<__half2*>(dst)[(c * 64 + 8 * bk + 2 * t4) / 2] =
-                    have_o ? __floats2half2_rn(__uint_as_float(o[c][4 * bk + 2 * half]) * sc,
-                                               __uint_as_float(o[c][4 * bk + 2 * half + 1]) * sc)
-                           : __floats2half2_rn(0.f, 0.f);
+                    __floats2half2_rn(__uint_as_float(o[c][4 * bk + 2 * half]) * sc,
+                                      __uint_as_float(o[c][4 * bk + 2 * half + 1]) * sc);
             }
           }
         }
@@ -986,9 +1003,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
               for (int bk = 0; bk < 8; ++bk)
                 *reinterpret_cast<float2*>(dst + c * 64 + 8 * bk + 2 * t4) =
-                    have_o ? make_float2(__uint_as_float(o[c][4 * bk + 2 * half]),
-                                         __uint_as_float(o[c][4 * bk + 2 * half + 1]))
-                           : make_float2(0.f, 0.f);
+                    make_float2(__uint_as_float(o[c][4 * bk + 2 * half]), __uint_as_float(o[c][4 * bk + 2 * half + 1]));
             }
           }
         }
@@ -999,8 +1014,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Pairs with the arrive after the prologue: every peer's receive barrier
     // is initialised.
     sm100::cluster_wait_acquire();
-    if (tid == 0) {
-      for (int c = 0; c < S; ++c) {
+    // (Four threads share the copies: one thread took about 100 cycles each.)
+    if (warp < kSoftmaxWarps && lane == 0) {
+      for (int c = warp; c < S; c += kSoftmaxWarps) {
         const int rc = max(0, min(nq, (c + 1) * rows_per) - c * rows_per);
         if (rc > 0)
           sm100::bulk_copy_to_cluster(sm100::mapa_shared(sm100::smem_addr(slots + split * rows_per * RS), c),

@@ -447,9 +447,18 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         // Keys past the prefix need no product (the rest of the last 16 are
         // zero in P and in V).
         const int ksteps = min(kChunk / 16, (chunk_keys(j) + 15) / 16);
-        for (int kk = 0; kk < ksteps; ++kk)
-          sm100::mma_bf16_ts(tmem + C::kOCol, a + kk * 8, sm100::smem_desc_sw128(v_addr + kk * 2048, C::kBlock, 1024),
-                             C::kIdescO, (j > 0 || kk > 0) ? 1u : 0u);
+        // (Whole chunks unrolled: 30.8 against 31.0 us at H = 32, Hkv = 8, KV
+        // 3500-6001.  Unrolled with a condition on every product: 32.7 us.)
+        const uint64_t vd = sm100::smem_desc_sw128(v_addr, C::kBlock, 1024);
+        sm100::mma_bf16_ts(tmem + C::kOCol, a, vd, C::kIdescO, j > 0 ? 1u : 0u);
+        if (ksteps == kChunk / 16) {
+#pragma unroll
+          for (int kk = 1; kk < kChunk / 16; ++kk)
+            sm100::mma_bf16_ts(tmem + C::kOCol, a + kk * 8, vd + kk * 128, C::kIdescO, 1u);
+        } else {
+          for (int kk = 1; kk < ksteps; ++kk)
+            sm100::mma_bf16_ts(tmem + C::kOCol, a + kk * 8, vd + kk * 128, C::kIdescO, 1u);
+        }
         sm100::mma_commit(sm100::smem_addr(&bars.done[j & 3]));
       }
       sm100::mma_commit(sm100::smem_addr(&bars.drain[1]));
