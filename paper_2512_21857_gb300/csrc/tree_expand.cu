@@ -3,8 +3,9 @@
 // adt_tree_rerank: the final top-N tree (Eq. 4 and the sentence after it).
 //
 // Expand is one launch of F thread-block clusters, one per frontier row; the
-// C <= 8 CTAs of a cluster split the row's vocabulary.  Each CTA stages its
-// share in shared memory with one bulk copy (x / T in fp32, round-to-nearest
+// C <= 8 CTAs of a cluster split the row's vocabulary.  Each CTA loads its
+// share into registers, eight logits a thread, or stages it in shared memory
+// with one bulk copy where it has more (x / T in fp32, round-to-nearest
 // division).  A first pass keeps each thread's largest value; the k-th
 // largest of the 32 warp maxima (64 half-warp maxima for k > 32) bounds the
 // CTA's top k from below; a second pass sums the exponentials against the
@@ -20,7 +21,7 @@
 //
 // A call is bound by the latency of that chain of phases, not by its bytes
 // (2.1 MB at F = 8, V = 65536: 0.3 us of HBM time).  Back-to-back calls in a
-// graph: 6.3 us at F = 8, V = 65536, k = 8 and 4.6 us at F = 1; 12.3 us at
+// graph: 5.6 us at F = 8, V = 65536, k = 8 and 4.0 us at F = 1; 10.4 us at
 // F = 39, V = 16384, k = 39 under guidance.  (With a bound that let half of a
 // CTA's logits through for k > 32, each of them inserted in sorted lists, the
 // last took 221.7 us.)
@@ -38,6 +39,7 @@ constexpr int kMaxCluster = 8;
 constexpr int kValuesPerCta = 2048;     // a CTA per this many logits, up to kMaxCluster per row
 constexpr int kTile = 32768;            // logits staged in shared memory at a time
 constexpr int kTileGuided = kTile / 2;  // under guidance (two rows)
+constexpr int kRegValues = 8;           // logits a thread of the register path holds
 constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr int kCandCap = 1024;          // a CTA's candidate buffer (also the cross-row keys)
 constexpr float kLog2e = 1.44269504088896340736f;
@@ -331,8 +333,14 @@ __device__ __forceinline__ void select_shared(const uint64_t* keys, int n, int k
 // The paths it leaves out are only code there, but a call is a chain of short
 // phases and each one fetched past them: with all of them a call at F = 8,
 // V = 65536, k = 8 took 0.4 us longer.
-template <bool kNarrow, bool kPlain>
-__global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) {
+// kRegs: the CTA's share is held in registers, from coalesced loads.  Staged in
+// shared memory instead (a bulk copy, its mbarrier, two passes of loads) the
+// calls took 6.3 against 5.6 us (F = 8, V = 65536, k = 8), 4.6 / 4.0 (F = 1),
+// 9.7 / 8.1 (F = 13, k = 13) and 12.3 / 10.4 (F = 39, V = 16384, k = 39,
+// guided).  A thread takes pairs: with vectors of four a share of 2048 logits
+// lies in half the warps, and their maxima bound a large k by nothing.
+template <bool kNarrow, bool kPlain, bool kRegs>
+__global__ void __launch_bounds__(kThreads, 1) expand_kernel(const ExpandParams p) {
   extern __shared__ __align__(16) float vals[];    // [min(per, tile)] staged logits (x2 with guidance)
   __shared__ uint64_t cand[kCandCap];              // keys at or above the CTA's bound
   __shared__ uint64_t wl[kWarps][kMaxK];           // overflow path: each warp's top k
@@ -360,7 +368,7 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   for (int i = tid; i < kMaxK; i += kThreads) ctl[i] = 0ull;
   if (tid == 0) {
     s_cnt = 0u;
-    sm100::mbar_init(sm100::smem_addr(&s_bar), 1);
+    if (!kRegs) sm100::mbar_init(sm100::smem_addr(&s_bar), 1);
     sm100::mbar_init(sm100::smem_addr(&s_push), 1);
     sm100::fence_mbar_init();
   }
@@ -370,10 +378,41 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   // This CTA's share of the row: [c0, c1), c0 a multiple of 4.
   const int per = (((p.V + C - 1) / C) + 3) & ~3;
   const int c0 = min(p.V, rank * per), c1 = min(p.V, c0 + per);
-  const int tile = kNarrow ? per : p.tile;
-  const int ntiles = kNarrow ? 1 : (c1 - c0 + tile - 1) / tile;
+  const int tile = kNarrow || kRegs ? per : p.tile;
+  const int ntiles = kNarrow || kRegs ? 1 : (c1 - c0 + tile - 1) / tile;
   const float* row = p.logits + static_cast<int64_t>(r) * p.ld;
   const float* row_u = p.logits_u ? p.logits_u + static_cast<int64_t>(r) * p.ld : nullptr;
+  float xr[kRegs ? kRegValues : 1];
+  auto reg_index = [&](int e) { return 2 * (tid + kThreads * (e / 2)) + e % 2; };  // of xr[e] in the share
+  if constexpr (kRegs) {
+    auto load = [&](const float* src, float* dst) {
+#pragma unroll
+      for (int u = 0; u < kRegValues / 2; ++u) {
+        const int i = reg_index(2 * u);
+        const float2 x = i < c1 - c0 ? __ldcg(reinterpret_cast<const float2*>(src + c0 + i))
+                                     : make_float2(-INFINITY, -INFINITY);
+        dst[2 * u] = x.x;
+        dst[2 * u + 1] = x.y;
+      }
+    };
+    load(row, xr);
+    if constexpr (!kPlain) {
+      if (row_u) {
+        float xu[kRegValues];
+        load(row_u, xu);
+#pragma unroll
+        for (int e = 0; e < kRegValues; ++e) xr[e] = adt::cfg_combine(xr[e], xu[e], p.cfg);
+      }
+      if (p.use_T) {
+#pragma unroll
+        for (int e = 0; e < kRegValues; ++e) xr[e] = __fdiv_rn(xr[e], p.T);
+      }
+    }
+    // Past the share's end (its last pair may hold one logit): no value.
+#pragma unroll
+    for (int e = 0; e < kRegValues; ++e)
+      if (reg_index(e) >= c1 - c0) xr[e] = -INFINITY;
+  }
   float* vals_u = vals + min(per, tile);  // used only with guidance
 
   // The row's frontier score and id, read now by the threads that write the
@@ -387,7 +426,11 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   // Pass 1: each thread's largest value.  Thread tid takes elements tid,
   // tid + 1024, ... of every tile.
   float v1 = -INFINITY;
-  for (int tt = 0; tt < ntiles; ++tt) {
+  if constexpr (kRegs) {
+#pragma unroll
+    for (int e = 0; e < kRegValues; ++e) v1 = fmaxf(v1, xr[e]);
+  }
+  for (int tt = 0; !kRegs && tt < ntiles; ++tt) {
     const int t0 = c0 + tt * tile, t1 = min(c1, t0 + tile);
     if (tt > 0) __syncthreads();  // the previous tile is consumed
     ok &= stage_tile<kPlain>(vals, vals_u, row, row_u, t0, t1, p, &s_bar, phase);
@@ -428,7 +471,18 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   // keys of values >= B (few: shared-memory atomics, no per-element vote).
   const float Ml = M == -INFINITY ? 0.f : M * kLog2e;
   float sa[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int tt = 0; tt < ntiles; ++tt) {
+  if constexpr (kRegs) {
+#pragma unroll
+    for (int e = 0; e < kRegValues; ++e) {
+      const int i = reg_index(e);
+      sa[e % 4] += ex2_approx(fmaf(xr[e], kLog2e, -Ml));
+      if (xr[e] >= B && i < c1 - c0) {
+        const unsigned pos = atomicAdd(&s_cnt, 1u);
+        if (pos < static_cast<unsigned>(kCandCap)) cand[pos] = adt::select_key(xr[e], static_cast<uint32_t>(c0 + i));
+      }
+    }
+  }
+  for (int tt = 0; !kRegs && tt < ntiles; ++tt) {
     const int t0 = c0 + tt * tile, t1 = min(c1, t0 + tile);
     if (ntiles > 1) {
       __syncthreads();
@@ -465,6 +519,14 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
     const uint64_t kb = B == -INFINITY ? 1ull : adt::select_key(B, 0xffffffffu);  // lowest key of value B
     WarpTopK tk;
     uint64_t thr = 0ull;
+    if constexpr (kRegs) {
+#pragma unroll
+      for (int e = 0; e < kRegValues; ++e) {
+        const int i = reg_index(e);
+        if (i < c1 - c0) vals[i] = xr[e];
+      }
+      __syncthreads();
+    }
     for (int tt = 0; tt < ntiles; ++tt) {
       const int t0 = c0 + tt * tile, t1 = min(c1, t0 + tile);
       if (ntiles > 1) {
@@ -625,7 +687,8 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
   if (tid == 0) *p.all_ticket = 0u;
 }
 
-// CTAs per row (the cluster size): one per kValuesPerCta logits, as long as
+// CTAs per row (the cluster size): at least kValuesPerCta logits each (a
+// share in registers has a pair for every thread), as long as
 // all rows' clusters run at once.  A CTA fills an SM (1024 threads of 63
 // registers) and the GPCs leave a part of the SMs out of a cluster's reach,
 // so the limit is four fifths of the SMs; beyond it the rows take two waves:
@@ -636,7 +699,7 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(const ExpandParams p) 
 // cut down stay even: three CTAs a row cost 9.0 against 7.6 us with two (F =
 // 39, guided).
 int expand_cluster(int F, int V, int sm_count) {
-  int c = (V + kValuesPerCta - 1) / kValuesPerCta;
+  int c = V / kValuesPerCta;
   c = c < 1 ? 1 : (c > kMaxCluster ? kMaxCluster : c);
   const int most = 4 * sm_count / (5 * F);
   if (c > most) c = most < 2 ? 1 : most / 2 * 2;
@@ -955,7 +1018,9 @@ static adt_status expand_impl(const float* logits, const float* logits_u, float 
   unsigned& word = configured[(info.device >> 5) & 1];
   const unsigned bit = 1u << (info.device & 31);
   if (!(__atomic_load_n(&word, __ATOMIC_ACQUIRE) & bit)) {
-    for (auto k : {expand_kernel<true, true>, expand_kernel<true, false>, expand_kernel<false, false>})
+    for (auto k : {expand_kernel<true, true, true>, expand_kernel<true, false, true>, expand_kernel<true, true, false>,
+                   expand_kernel<true, false, false>, expand_kernel<false, false, true>,
+                   expand_kernel<false, false, false>})
       ADT_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(kTile * sizeof(float))));
     __atomic_fetch_or(&word, bit, __ATOMIC_ACQ_REL);
@@ -976,8 +1041,15 @@ static adt_status expand_impl(const float* logits, const float* logits_u, float 
   const bool narrow = k_child <= kThreads / 16 / kMaxCluster && per <= p.tile &&
                       (!keep_idx || F * k_child <= kThreads / 16);
   const bool plain = !logits_u && !p.use_T;
-  ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, !narrow ? expand_kernel<false, false>
-                                        : plain ? expand_kernel<true, true> : expand_kernel<true, false>, p));
+  // A pair in every thread (the bound needs values in all warps) up to eight
+  // logits a thread.
+  const bool regs = per >= 2 * kThreads && per <= kRegValues * kThreads;
+  auto kernel = narrow ? (plain ? expand_kernel<true, true, false> : expand_kernel<true, false, false>)
+                       : expand_kernel<false, false, false>;
+  if (regs)
+    kernel = narrow ? (plain ? expand_kernel<true, true, true> : expand_kernel<true, false, true>)
+                    : expand_kernel<false, false, true>;
+  ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, p));
   return adt::launch_status();
 }
 

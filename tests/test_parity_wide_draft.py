@@ -132,3 +132,22 @@ def test_expand_scores_outside_the_range_of_fp32(V, k, mask):
             np.testing.assert_allclose(got["child_logp"][sl], lp.astype(np.float32), rtol=1e-6, atol=1e-6)
             np.testing.assert_allclose(got["child_score"][sl], (float(fscore[r]) + lp).astype(np.float32),
                                        rtol=1e-6, atol=1e-6)
+
+
+@pytest.mark.parametrize("k", [8, 39])
+@pytest.mark.parametrize("F,V", [(2, 2047), (2, 2048), (2, 2049), (3, 4097), (2, 65533), (2, 65536), (2, 65540),
+                                 (16, 65536)])
+def test_expand_share_in_registers(F, V, k):
+    """Shares of one pair a thread to eight logits a thread, an odd logit at
+    the end, and one logit less or more a share than registers are used for
+    (2047; 8193 of 65540; 10924 in six CTAs), plain, divided by a temperature
+    and guided."""
+    logits = synth.f32_normal((F, V), V + k, "logits", std=3.0)
+    fscore = synth.f32_normal((F,), V, "fs", std=1.0)
+    keep = min(F * k, 64)
+    for T in (1.0, 0.7):
+        got, _ = run_expand(logits, fscore, None, k, keep, T=T)
+        check_expand(got, oracle.tree_expand(logits, fscore, k, keep, temperature=T), keep)
+    cond, uncond = (synth.f32_normal((F, V), V + i, "l", std=3.0) for i in range(2))
+    got = run_expand_cfg(cond, uncond, fscore, None, k, keep)
+    check_expand(got, oracle.tree_expand(oracle.cfg_logits(cond, uncond, 3.0), fscore, k, keep), keep)
