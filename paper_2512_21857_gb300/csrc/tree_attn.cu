@@ -40,7 +40,7 @@
 // splits they merge through the workspace.
 //
 // Back-to-back launches at the 7B shape (four splits, 41.4 MB, 6.1 us at the
-// measured HBM rate) take 12.5 us, at the LlamaGen shape (six splits, from L2)
+// measured HBM rate) take 11.3 us, at the LlamaGen shape (six splits, from L2)
 // 7.1 us: the chain from the dependency wait through the first loads to the
 // merge, whose instructions come cold for each launch.  So one copy of the
 // softmax serves every chunk, masks are bit tests on one word per row, the
@@ -50,13 +50,15 @@
 // alone, and four threads send the merge's rows (7.3 us without).  One split
 // writes its rows directly (eight ragged trees, 41.9 -> 38.4 us a layer).
 //
-// Where the 7B launch's 11 us from the dependency wait to the end go (cycles
-// at 1.93 GHz): 1500 to the first load, 4000 to the first K tile (every CTA's
-// first 128 KB at once), 8800 for the stream (6.3 TB/s), then 1700 for the last
-// softmax, 1800 for its PV product, 1000 to write the partial rows, 1900 to
-// move them, 800 to merge.  Requests ahead of the ring (L2 prefetches of the
-// next chunks, or of the first ones before the dependency wait) made it slower
-// or no faster (12.5-13.5 us): they delay the tiles that are needed first.
+// Where the 7B launch's 11 us from the dependency wait to the end went before
+// its first chunks were prefetched (cycles at 1.93 GHz): 1500 to the first load,
+// 4000 to the first K tile (every CTA's first 128 KB at once), 8800 for the
+// stream (6.3 TB/s), then 1700 for the last softmax, 1800 for its PV product,
+// 1000 to write the partial rows, 1900 to move them, 800 to merge.  Spare
+// clusters now prefetch during those last phases of the launch before (see
+// prefetch_stream, 12.5 -> 11.3 us); prefetches by the CTAs that compute made it
+// slower or no faster (12.5-13.5 us): they delay the tiles that are needed
+// first.
 //
 // Launches with long key ranges per CTA whose tiles can hold more than 64 rows
 // (trees of more than 64 nodes, grouped query heads) take the 128-row kernel
@@ -142,6 +144,7 @@ struct TcParams {
   const int32_t* parents;
   const int32_t* offs;
   int B, H, Hkv, group, max_kv, splits;
+  int prefetch;       // leading blockIdx.y rows of clusters that only prefetch (see prefetch_stream)
   int qtiles;         // 64-row query tiles per tree: ceil(max_nodes / 64)
   int cluster_merge;
   int max_tree;       // largest tree accepted: 64 * qtiles
@@ -366,6 +369,50 @@ __device__ __forceinline__ TreeSlot tree_of_slot(const TcParams& p, int slot, in
   return t;
 }
 
+// A launch whose clusters leave SMs free puts further clusters on them, which
+// bring the first kPrefetchChunks chunks of every split into L2 and end.  They
+// run ahead of the dependency wait, while the launch before finishes (its
+// merge leaves the memory idle), so what they read are hints: kv_len may be
+// about to change, and the lines they touch lie in the cache tensor whatever
+// it says (the tensor map bounds them; later writes go through the same L2).
+// A thread asks for one box of 128 keys x 64 columns, chunk by chunk over the
+// CTAs; an SM's requests go out at about 115 GB/s, so a CTA takes at most 1.5
+// MB.  The launch before lets them start once it has requested its last K
+// tiles (started at once, they take bandwidth from its own stream).
+//
+// us a layer back to back, D = 128, without and with: H = 32, KV 2400 12.5 and
+// 11.3, KV 1200 9.8 and 9.2, KV 4096 16.5 and 15.9; H = 16, KV 2400 10.3 and 9.8;
+// H = 24 11.3 and 11.2; four trees of KV 2320 30.5 and 30.2; in the 128-row
+// kernel 256 nodes, KV 2400 19.2 and 18.6, four trees, Hkv = 8, KV 3500-6001
+// 30.6 and 30.0.  One or two chunks gave half of it, all chunks took longer
+// than none (14.6 us for the first).
+constexpr int kPrefetchChunks = 3;
+constexpr int kPrefetchBoxes = 96;  // a CTA's share: 1.5 MB
+
+// Tree b's prefix of L keys: split s of S takes chunks s W / S and on of the W
+// (tree chunks, which the kernels count as tree_chunks, follow the prefix).
+template <int kBlocks>
+__device__ __noinline__ void prefetch_stream(const CUtensorMap* tm_k, const CUtensorMap* tm_v, const TcParams& p, int b,
+                                             int S, int tree_chunks) {
+  const int L = min(max(__ldcg(p.kv_len + b), 0), p.max_kv);
+  const int Pc = (L + kChunk - 1) / kChunk, W = Pc + tree_chunks;
+  const int per = p.Hkv * S * 2 * kBlocks;  // column blocks of one chunk of every split, K and V
+  const int w = (static_cast<int>(threadIdx.x) * p.prefetch + static_cast<int>(blockIdx.y)) *
+                    static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);
+  if (threadIdx.x >= kPrefetchBoxes || w >= per * kPrefetchChunks) return;
+  const int blk = w % kBlocks, v = w / kBlocks % 2, pair = w % per / (2 * kBlocks);
+  const int split = pair % S, c = split * W / S + w / per;
+  if (c < min((split + 1) * W / S, Pc))
+    sm100::tma_prefetch_4d(v ? tm_v : tm_k, blk * 64, c * kChunk, pair / S, b);
+}
+
+// Clusters that prefetch: what the compute clusters of a launch leave of the
+// clusters that fit at once, evenly over its trees, up to eight a tree.
+int prefetch_clusters(int fit, int compute, int per_tree) {
+  const int room = (fit - compute) / per_tree;
+  return room < 0 ? 0 : room > 8 ? 8 : room;
+}
+
 // kLarge: trees of more than 64 nodes (query tiles, one mask word per tree
 // unit); otherwise one tile and one word, kept in registers.
 
@@ -388,13 +435,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int s_last;
   __shared__ volatile int s_abort;
 
-  const int split = blockIdx.x, h = blockIdx.y;
+  constexpr bool kPrefetch = D == 128 && !kLarge;
+  const int split = blockIdx.x, h = static_cast<int>(blockIdx.y) - (kPrefetch ? p.prefetch : 0);
   const int slot = kLarge ? static_cast<int>(blockIdx.z) / p.qtiles : static_cast<int>(blockIdx.z);
   const int qt = kLarge ? static_cast<int>(blockIdx.z) % p.qtiles : 0;
   const int g = h / p.group;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = C::kStages;
 
+  if (kPrefetch && h < 0) {
+    prefetch_stream<C::kBlocks>(&tm_k, &tm_v, p, static_cast<int>(blockIdx.z), p.splits, 1);
+    return;
+  }
   // Set-up that touches no memory the previous kernel writes: the
   // mbarriers, the tensor memory and the tensor maps' descriptors.  It runs
   // before the dependency wait, so a CTA that is resident early (on an SM
@@ -666,6 +718,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         issue_tile(j);
         ++issued;
       }
+      // With its last K tile requested, a next launch may start to prefetch.
+      if (kPrefetch && p.prefetch && !load_v) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
       // Every copy issued lands before the CTA goes on: after an abort
       // elsewhere its consumer may never have waited for it (on the normal
       // path these waits return at once).
@@ -1446,7 +1500,14 @@ adt_status launch(TcParams prm, const void* k_cache, const void* v_cache, int64_
   if ((s1 = make_rows_map(&tm_vt, prm.vt, D, prm.Hkv)) != ADT_OK) return s1;
   prm.cluster_merge = prm.splits <= kMaxClusterSplits ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(prm.splits), static_cast<unsigned>(prm.H),
+  // At least 2.5 chunks a split: a launch of less is mostly latency.  At D = 64,
+  // where a chunk is half the bytes, there is no gain (H = 20, KV 2400: 9.8 and
+  // 9.8 us; in the 128-row kernel 12.4 and 12.4 us, 192 nodes, KV 693 and 577).
+  prm.prefetch = 0;
+  if (D == 128 && !kLarge && overlap_previous && prm.cluster_merge &&
+      2 * ((prm.max_kv + kChunk - 1) / kChunk + 1) >= 5 * prm.splits)
+    prm.prefetch = prefetch_clusters(max_active_clusters(D, kLarge, prm.splits, dev), prm.B * prm.H, prm.B);
+  cfg.gridDim = dim3(static_cast<unsigned>(prm.splits), static_cast<unsigned>(prm.H + prm.prefetch),
                      static_cast<unsigned>(prm.B * prm.qtiles));
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = Cfg<D>::kDynSmem;
@@ -1522,7 +1583,11 @@ adt_status launch_wide(TcParams prm, int heads, const void* k_cache, const void*
   const int groups = prm.B * (prm.H / heads);
   const int cluster = wide_cluster<D>(sm_count, groups, tiles, prm.max_kv, dev);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(prm.H / heads),
+  prm.prefetch = 0;
+  if (D == 128 && overlap_previous)
+    prm.prefetch = prefetch_clusters(wide_active_clusters<D>(cluster, dev), groups * (cluster > 1 ? 1 : tiles),
+                                     prm.B * (cluster > 1 ? 1 : tiles));
+  cfg.gridDim = dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(prm.H / heads + prm.prefetch),
                      static_cast<unsigned>(cluster > 1 ? prm.B : prm.B * tiles));
   cfg.blockDim = dim3(kWideThreads, 1, 1);
   cfg.dynamicSmemBytes = WideCfg<D>::kDynSmem;
