@@ -40,13 +40,13 @@
 // splits they merge through the workspace.
 //
 // Back-to-back launches at the 7B shape (four splits, 41.4 MB, 6.1 us at the
-// measured HBM rate) take 11.3 us, at the LlamaGen shape (six splits, from L2)
-// 7.1 us: the chain from the dependency wait through the first loads to the
-// merge, whose instructions come cold for each launch.  So one copy of the
-// softmax serves every chunk, masks are bit tests on one word per row, the
+// measured HBM rate) take 11.3 to 11.8 us, at the LlamaGen shape (six splits,
+// from L2) 7.1 us: the chain from the dependency wait through the first loads
+// to the merge, whose instructions come cold for each launch.  So one copy of
+// the softmax serves every chunk, masks are bit tests on one word per row, the
 // merge is unrolled for the split count's range, and paths off the common one
-// lie behind it (12.9 and 7.4 us with two softmax copies, 64-bit masks and an
-// eight-way merge inline); the first S product waits for the tensor copies
+// lie behind it (7.4 us at the LlamaGen shape with two softmax copies, 64-bit
+// masks and an eight-way merge inline); the first S product waits for the tensor copies
 // alone, and four threads send the merge's rows (7.3 us without).  One split
 // writes its rows directly (eight ragged trees, 41.9 -> 38.4 us a layer).
 //
@@ -484,9 +484,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   sm100::tc_fence_after();
   const uint32_t tmem = tmem_slot;
 
-  // Programmatic dependent launch: every global-memory access comes after
-  // the previous kernel in the stream has completed (immediate when this
-  // launch does not overlap one).
+  // Programmatic dependent launch: every global-memory access that a result
+  // depends on comes after the previous kernel in the stream has completed
+  // (immediate when this launch does not overlap one).
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   const TreeSlot ts = tree_of_slot(p, slot, lane);
   const int b = ts.b, node0 = ts.node0, n = ts.n, total_nodes = ts.total_nodes, L = ts.L;
@@ -1548,8 +1548,8 @@ int wide_cluster(int sm_count, int groups, int tiles, int max_kv, int dev) {
 // thread per row): it pays from about kWideChunks chunks per CTA of the 64-row
 // kernel on.  64-row / 128-row kernel, us: two chunks (H = 8 / 2, D = 64, four
 // trees over 600 keys) 8.8 / 9.6, three (20 / 5 heads, D = 64, 2400 keys)
-// 10.6 / 11.1, nine (32 / 8, D = 128, 4000 keys) 15.3 / 13.2, 20 (256 nodes,
-// 32 heads, D = 128, 2400 keys) 29.9 / 19.1.
+// 10.6 / 11.1, nine (32 / 8, D = 128, 4000 keys) 15.3 / 13.1, 20 (256 nodes,
+// 32 heads, D = 128, 2400 keys) 29.9 / 18.6.
 constexpr int kWideChunks = 6;
 
 int wide_heads(const TcParams& prm, int sm_count) {

@@ -26,8 +26,8 @@
 // chunk the latency of a group's turn (2600 cycles for scores to
 // probabilities, two groups at a time) beside 64 KB of K and V a CTA (11 TB/s
 // from L2 over all CTAs).  Per layer, the 64-row kernel before: 256 nodes, 32
-// heads x 128, 2400 keys 29.9 -> 19.1 us; four trees of 33 to 64 nodes, 32 / 8
-// heads x 128, 3500 to 6001 keys 54.1 -> 30.6 us; two trees of 192 nodes, 20 heads x 64,
+// heads x 128, 2400 keys 29.9 -> 18.6 us; four trees of 33 to 64 nodes, 32 / 8
+// heads x 128, 3500 to 6001 keys 54.1 -> 30.0 us; two trees of 192 nodes, 20 heads x 64,
 // 693 and 577 keys 15.1 -> 12.3 us; 41 nodes in a call sized for 256, 32 heads
 // x 128, 1203 keys 18.2 -> 10.2 us.  One accumulator and P apart from S (so
 // that the next scores do not wait for the PV product) took the first from
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (sm100::smem_addr(smem_raw) & 1023u)) & 1023u);
   __shared__ WideBarriers bars;
-  __shared__ __align__(16) uint32_t anc[kWideRows][2 * kMaxTreeUnits];  // ancestor bits of the tile's nodes, 32 nodes a word
+  __shared__ __align__(16) uint32_t anc[kWideRows][2 * kMaxTreeUnits];  // ancestor bits of the tile's nodes
   __shared__ int s_par[kMaxTreeNodes];
   __shared__ float s_mu[kWideRows];
   __shared__ float2 s_ml[2][kWideRows];
