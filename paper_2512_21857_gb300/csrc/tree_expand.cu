@@ -36,7 +36,6 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxK = 64;
 constexpr int kMaxKeep = 1024;
 constexpr int kMaxCluster = 8;
-constexpr int kValuesPerCta = 2048;     // a CTA per this many logits, up to kMaxCluster per row
 constexpr int kTile = 32768;            // logits staged in shared memory at a time
 constexpr int kTileGuided = kTile / 2;  // under guidance (two rows)
 constexpr int kRegValues = 8;           // logits a thread of the register path holds
@@ -687,22 +686,26 @@ __global__ void __launch_bounds__(kThreads, 1) expand_kernel(const ExpandParams 
   if (tid == 0) *p.all_ticket = 0u;
 }
 
-// CTAs per row (the cluster size): at least kValuesPerCta logits each (a
-// share in registers has a pair for every thread), as long as
-// all rows' clusters run at once.  A CTA fills an SM (1024 threads of 63
-// registers) and the GPCs leave a part of the SMs out of a cluster's reach,
-// so the limit is four fifths of the SMs; beyond it the rows take two waves:
-// F = 39, V = 16384, k = 39, without the next frontier: 15.7, 13.2, 11.4, 6.9
-// and 7.6 us with 8, 6, 4, 2 and 1 CTAs per row; F = 20, k = 20: 10.6, 6.1,
-// 6.0, 6.2 and 7.3 us; at V = 65536 14.4, 12.1 and 18.5 us with 4, 2 and 1
-// (F = 39) and 12.0, 7.1, 7.3 and 11.4 with 8, 6, 4 and 2 (F = 20).  Sizes
-// cut down stay even: three CTAs a row cost 9.0 against 7.6 us with two (F =
-// 39, guided).
-int expand_cluster(int F, int V, int sm_count) {
-  int c = V / kValuesPerCta;
-  c = c < 1 ? 1 : (c > kMaxCluster ? kMaxCluster : c);
+// CTAs per row (the cluster size).  A share of 8192 logits is the most that
+// registers hold; with up to 8 children half of that is a little faster, with
+// more of them every CTA more means a longer list to rank (us with 8, 4 and 2
+// CTAs at V = 16384: F = 8, k = 8 5.6, 5.7, 5.7; F = 13, k = 13 8.0, 7.5, 7.5; F =
+// 1, k = 39, guided 6.6, 6.3, 5.5; F = 20, k = 20, no next frontier 8.3, 4.6,
+// 4.3).  All rows' clusters run at once: a CTA fills an SM (1024 threads) and
+// the GPCs leave a part of the SMs out of a larger cluster's reach, so the
+// limit is four fifths of the SMs for those, and all of them for pairs; beyond
+// it the rows take two waves (F = 20, V = 65536, 8, 6 and 4 CTAs: 8.8, 6.9, 7.2;
+// F = 39 with 4, 3 and 2: 15.0, 9.9, 10.2; F = 76, V = 32768 with 2 and 1: 5.8,
+// 7.1, F = 90 11.0, 7.7).  Sizes cut down stay even (F = 39, V = 16384, guided,
+// 3 and 2: 12.2 and 10.5).
+int expand_cluster(int F, int V, int k, int sm_count) {
+  const int share = k <= 8 ? kRegValues * kThreads / 2 : kRegValues * kThreads;
+  int c = (V + share - 1) / share;
+  const int pairs = V / (2 * kThreads);  // shares that still have a pair of logits for each thread
+  if (c < 2) c = pairs < 2 ? 1 : 2;
+  if (c > kMaxCluster) c = kMaxCluster;
   const int most = 4 * sm_count / (5 * F);
-  if (c > most) c = most < 2 ? 1 : most / 2 * 2;
+  if (c > most) c = most >= 2 ? most / 2 * 2 : c > 1 && 2 * F <= sm_count ? 2 : 1;
   return c;
 }
 
@@ -1010,7 +1013,7 @@ static adt_status expand_impl(const float* logits, const float* logits_u, float 
   p.cross_keys = reinterpret_cast<uint64_t*>(ws + w.cross_keys);
   p.all_ticket = reinterpret_cast<unsigned*>(ws + w.all_ticket);
   p.err = info.error_word;
-  const int C = expand_cluster(F, V, info.sm_count);
+  const int C = expand_cluster(F, V, k_child, info.sm_count);
   const int per = ((V + C - 1) / C + 3) & ~3;
   p.tile = logits_u ? kTileGuided : kTile;
   const size_t dyn = static_cast<size_t>(per < p.tile ? per : p.tile) * sizeof(float) * (logits_u ? 2 : 1);

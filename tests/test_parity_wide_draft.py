@@ -136,12 +136,13 @@ def test_expand_scores_outside_the_range_of_fp32(V, k, mask):
 
 @pytest.mark.parametrize("k", [8, 39])
 @pytest.mark.parametrize("F,V", [(2, 2047), (2, 2048), (2, 2049), (3, 4097), (2, 65533), (2, 65536), (2, 65540),
-                                 (16, 65536)])
+                                 (16, 65536), (64, 16384), (77, 4096)])
 def test_expand_share_in_registers(F, V, k):
     """Shares of one pair a thread to eight logits a thread, an odd logit at
     the end, and one logit less or more a share than registers are used for
-    (2047; 8193 of 65540; 10924 in six CTAs), plain, divided by a temperature
-    and guided."""
+    (2047; 8196 of 65540; 10924 in six CTAs), rows in pairs of CTAs and, one
+    row more than pairs of SMs, in single ones; plain, divided by a
+    temperature and guided."""
     logits = synth.f32_normal((F, V), V + k, "logits", std=3.0)
     fscore = synth.f32_normal((F,), V, "fs", std=1.0)
     keep = min(F * k, 64)
