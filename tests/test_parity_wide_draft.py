@@ -152,3 +152,33 @@ def test_expand_share_in_registers(F, V, k):
     cond, uncond = (synth.f32_normal((F, V), V + i, "l", std=3.0) for i in range(2))
     got = run_expand_cfg(cond, uncond, fscore, None, k, keep)
     check_expand(got, oracle.tree_expand(oracle.cfg_logits(cond, uncond, 3.0), fscore, k, keep), keep)
+
+
+@pytest.mark.parametrize("F,V,k", [
+    (8, 65536, 8), (8, 16384, 39),  # shares in registers: narrow and general instantiation
+    (8, 2047, 8), (8, 2047, 39),    # staged in shared memory
+    (130, 40000, 9),                # two tiles
+])
+def test_expand_rows_of_any_magnitude(F, V, k):
+    """Rows that lie wholly at fp32's lowest value, near it, around +-1e10 and
+    2^20, beside ordinary ones: log-probabilities are those of fp64 (-ln V where all
+    logits are equal), and such a row does not disturb the next frontier."""
+    logits = synth.f32_normal((F, V), V + k, "logits", std=3.0)
+    for r, level in ((1, LOWEST), (2, -3e38), (3, -1e10), (4, 1e10), (5, 3e38)):
+        logits[r] = np.float32(level)
+    logits[4, 5:V:7] = np.nextafter(np.float32(1e10), np.float32(0))  # 1024 below: no weight
+    logits[0] += np.float32(2 ** 20 - 64)  # terms of either form
+    logits[6] += np.float32(2 ** 20)
+    fscore = synth.f32_normal((F,), V, "fs", std=1.0)
+    got, _ = run_expand(logits, fscore, None, k, k)
+    for r in range(F):
+        x = logits[r].astype(np.float64)
+        m = x.max()
+        order = np.argsort(-x, kind="stable")[:k]
+        lp = x[order] - m - np.log(np.exp(x - m).sum())
+        sl = slice(r * k, (r + 1) * k)
+        assert got["child_token"][sl].tolist() == order.tolist()
+        np.testing.assert_allclose(got["child_logp"][sl], lp.astype(np.float32), rtol=1e-6, atol=1e-6)
+        np.testing.assert_allclose(got["child_score"][sl], (float(fscore[r]) + lp).astype(np.float32), rtol=1e-6,
+                                   atol=1e-6)
+    assert got["keep_idx"].tolist() == np.argsort(-got["child_score"], kind="stable")[:k].tolist()
