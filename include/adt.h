@@ -104,15 +104,17 @@ adt_status adt_get_device_error(void* stream, uint32_t* bits);
 const char* adt_status_string(adt_status s);
 
 /* Testing hook, not for production use.  Every wait of adt_tree_attn's
- * pipeline (a CTA waiting for its loads, products or softmax stages) is
- * bounded: after `polls` unsuccessful polls it gives up, sets
+ * pipeline (a CTA waiting for its loads, products or softmax stages) and of
+ * adt_tree_accept's sampling walks (a CTA waiting for its cluster's values)
+ * is bounded: after `polls` unsuccessful polls it gives up, sets
  * ADT_DEVERR_TIMEOUT in the device error word and the kernel leaves cleanly
- * (the copies and tensor-core products it already issued are waited for
- * first, so the device stays usable; the outputs of that call are
- * unspecified).  This sets the bound for the launches that follow in this
- * process; 0 restores the default (2^20 polls).  It lets a test make a
- * bounded wait run out without any fault; it is not synchronised with
- * calls on other threads. */
+ * (the copies and tensor-core products it already issued, and the stores to
+ * it that are on their way, are waited for first, so the device stays usable;
+ * the outputs of that call are unspecified).  This sets the bound for the
+ * launches that follow in this process; 0 restores the defaults (2^20 and
+ * 2^22 polls), 1 makes every wait of a sampling walk give up.  It lets a
+ * test make a bounded wait run out without any fault; it is not synchronised
+ * with calls on other threads. */
 adt_status adt_testing_set_wait_limit(uint32_t polls);
 
 /* Testing hook, not for production use: out[i] = e^(a[i] - b[i]) (a[i] <= b[i])

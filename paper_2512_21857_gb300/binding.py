@@ -165,7 +165,7 @@ def adt_get_device_error(stream=None) -> int:
 
 
 def adt_testing_set_wait_limit(polls: int) -> None:
-    """Testing hook: polls before adt_tree_attn's pipeline waits give up (0 = default)."""
+    """Testing hook: polls before the waits of adt_tree_attn and of sampling walks give up (0 = defaults)."""
     _check(lib().adt_testing_set_wait_limit(int(polls)), "adt_testing_set_wait_limit")
 
 

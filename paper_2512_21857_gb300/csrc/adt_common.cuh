@@ -32,6 +32,10 @@ struct DeviceInfo {
 // Cached per device; thread-safe.  Returns ADT_ERR_CUDA when the runtime fails.
 adt_status device_info(DeviceInfo* out);
 
+// Polls before a kernel's bounded wait gives up: kernel_limit, or what
+// adt_testing_set_wait_limit set.
+uint32_t wait_limit(uint32_t kernel_limit);
+
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

@@ -29,9 +29,18 @@ void init_device(int dev) {
   g_info_status[dev] = ADT_OK;
 }
 
+// Polls before a bounded wait gives up; 0: the kernels' own limits.  Set only
+// by adt_testing_set_wait_limit.
+uint32_t g_wait_limit = 0;
+
 }  // namespace
 
 namespace adt {
+
+uint32_t wait_limit(uint32_t kernel_limit) {
+  const uint32_t lim = __atomic_load_n(&g_wait_limit, __ATOMIC_RELAXED);
+  return lim ? lim : kernel_limit;
+}
 
 adt_status device_info(DeviceInfo* out) {
   int dev = 0;
@@ -60,6 +69,11 @@ const char* adt_status_string(adt_status s) {
     case ADT_ERR_DEVICE: return "ADT_ERR_DEVICE";
   }
   return "ADT_ERR_UNKNOWN";
+}
+
+adt_status adt_testing_set_wait_limit(uint32_t polls) {
+  __atomic_store_n(&g_wait_limit, polls, __ATOMIC_RELAXED);
+  return ADT_OK;
 }
 
 adt_status adt_get_device_error(void* stream, uint32_t* bits) {

@@ -40,7 +40,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxNodes = 1024;
 constexpr int kMostCtas = 16;      // per tree
 constexpr int kBatch = 64;         // children of a node taken out of the slices together
-constexpr uint32_t kWaitLimit = 1u << 22;
+constexpr uint32_t kWaitLimit = 1u << 22;   // polls
+constexpr uint32_t kLandLimit = 1u << 12;   // polls (of 10 ns and more) for stores on their way
 
 struct AcceptParams {
   const float* target;
@@ -65,6 +66,7 @@ struct AcceptParams {
   int32_t* alen;
   int32_t* bonus;
   unsigned* err;
+  uint32_t wait_limit;  // polls before a wait gives up
   int Vs;  // vocabulary slice per CTA (multiple of 4)
 };
 
@@ -80,6 +82,13 @@ struct Tree {
   int nkids;
   int bad;
 };
+
+// What a tree that is skipped gets: the root alone.  One thread.
+__device__ void write_skipped(const AcceptParams& p, int b) {
+  p.alen[b] = 0;
+  p.bonus[b] = 0;
+  for (int i = 0; i < p.max_path; ++i) p.path[static_cast<int64_t>(b) * p.max_path + i] = i == 0 ? 0 : -1;
+}
 
 // Parents and tokens of tree b into shared memory; false, with the error
 // raised and the outputs set (by the cluster's first CTA), for a malformed
@@ -101,9 +110,7 @@ __device__ bool load_tree(Tree* t, const AcceptParams& p, int b, int node0, int 
   if (!t->bad) return true;
   if (first && tid == 0) {
     adt::raise_error(p.err, ADT_DEVERR_BAD_TREE);
-    p.alen[b] = 0;
-    p.bonus[b] = 0;
-    for (int i = 0; i < p.max_path; ++i) p.path[static_cast<int64_t>(b) * p.max_path + i] = i == 0 ? 0 : -1;
+    write_skipped(p, b);
   }
   return false;
 }
@@ -379,10 +386,16 @@ __device__ __forceinline__ dfl::df resid(dfl::df ep, dfl::df eq, dfl::df B) {
 // the children's) goes on.  Two rounds' entries are kept apart by the round's
 // parity: a warp pushes for round r + 2 only once round r + 1 is complete, for
 // which every warp of the cluster has pushed after it was done with round r.
+//
+// A wait that runs out raises the error and sets `late` in its thread.  The
+// block barrier that follows every wait, before anything else is pushed, tells
+// the others: the walk ends there, and the CTA pushes no more.
 struct Rounds {
   SampleShared* sh;
   unsigned* err;
+  uint32_t limit;
   int rank, csize, r;
+  int late;
   __device__ __forceinline__ void send(float4 v, const void* local, int c) {
     asm volatile(
         "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n" ::"r"(
@@ -398,9 +411,23 @@ struct Rounds {
       sm100::mbar_arrive_expect_tx(sm100::smem_addr(&sh->bar[r & 1]),
                                    static_cast<uint32_t>(csize * kWarps * sizeof(float4) + extra));
   }
+  __device__ __forceinline__ bool poll(uint32_t polls) {
+    return sm100::mbar_wait_bounded(sm100::smem_addr(&sh->bar[r & 1]), (r >> 1) & 1, polls);
+  }
   __device__ __forceinline__ void wait() {
-    if (!sm100::mbar_wait_bounded(sm100::smem_addr(&sh->bar[r & 1]), (r >> 1) & 1, kWaitLimit))
+    if (!poll(limit)) {
       adt::raise_error(err, ADT_DEVERR_TIMEOUT);
+      late = 1;
+    }
+  }
+  // The end of a CTA with a late wait: peers may still push to it (those that
+  // are not late have all they wait for and may be gone).  It stays until every
+  // peer has ended or come here too, so that none pushes any more, and for the
+  // stores that are on their way.
+  __device__ __forceinline__ void stay() {
+    sm100::cluster_arrive_release();
+    sm100::cluster_wait_acquire();
+    (void)poll(kLandLimit);
   }
   __device__ __forceinline__ const float4* entries() const { return sh->part[r & 1]; }
   __device__ __forceinline__ int count() const { return csize * kWarps; }
@@ -493,7 +520,7 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
   sm100::cluster_arrive_release();  // the mbarriers are there: waited for before the first push
   adt::pdl_wait_then_release();
   cg::cluster_group cl = cg::this_cluster();
-  Rounds rd{&sh, p.err, static_cast<int>(cl.block_rank()), static_cast<int>(cl.num_blocks()), 0};
+  Rounds rd{&sh, p.err, p.wait_limit, static_cast<int>(cl.block_rank()), static_cast<int>(cl.num_blocks()), 0, 0};
   const int b = blockIdx.x / rd.csize;
   E* pbuf = reinterpret_cast<E*>(dyn);
   E* qbuf = pbuf + p.Vs;
@@ -549,6 +576,7 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
     int nxt = -1;
     dfl::df N{0.f, 0.f}, B{0.f, 0.f};  // SPEC, warp 0 (N = 0: not set yet)
     bool exps = false;                 // the slices hold exponentials
+    int late = 0;                      // the same in every thread
     for (int base = 0; nxt < 0 && (base < nk || !exps); base += kBatch) {
       const int nb = min(kBatch, max(0, nk - base));
       // The batch's tokens leave the slices.
@@ -559,7 +587,8 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
       }
       if (tid < nb) sh.kid_tok[tid] = tree.tok[tree.kids[base + tid]];
       if (tid == 0) sh.tree_own = 0;
-      __syncthreads();  // also: this CTA's slices are written
+      late = __syncthreads_or(rd.late);  // also: this CTA's slices are written
+      if (late) break;
       if (tid < nb) {
         const int x = sh.kid_tok[tid];
         int rep = tid;
@@ -662,7 +691,8 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
               if (sh.kid_state[j] == 4) adt::raise_error(p.err, ADT_DEVERR_BAD_INDEX);
           if (lane == 0) sh.bi[0] = at;
         }
-        __syncthreads();
+        late = __syncthreads_or(rd.late);
+        if (late) break;
         if (sh.bi[0] < nb) nxt = tree.kids[base + sh.bi[0]];
       } else {
         // Q and 1 / Q once the children before this one are gone.
@@ -715,7 +745,8 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
               sh.bf[0] = make_float2(nB.hi, nB.lo);
             }
           }
-          __syncthreads();
+          late = __syncthreads_or(rd.late);
+          if (late) break;
           const int verdict = sh.bi[0];
           if (verdict == 1) nxt = tree.kids[base + sh.bi[1]];
           if (verdict != 2) break;
@@ -768,6 +799,7 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
           }
           ++rd.r;
         }
+        if (late) break;
         if (nxt < 0) {
           // All of the batch rejected: their tokens return to the slices.
           if (warp == 0) {
@@ -792,7 +824,7 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
       // slice and reads it starting at offset t mod its length, wrapping
       // around: at the same step the threads of a half-warp then touch
       // different banks.
-      __syncthreads();
+      if (late || __syncthreads_or(rd.late)) break;
       const dfl::df fB{sh.bf[1].x, sh.bf[1].y};
       const int per = (cnt + kThreads - 1) / kThreads;
       const int b0 = min(cnt, tid * per), b1 = min(cnt, b0 + per), len = b1 - b0;
@@ -877,10 +909,14 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
     v = nxt;
     __syncthreads();  // the node's lists are rewritten
   }
-  __syncthreads();
+  if (__syncthreads_or(rd.late)) {
+    if (rd.rank == 0 && tid == 0) write_skipped(p, b);
+    rd.stay();
+    return;
+  }
   if (rd.rank == 0) write_path(&tree, p, b, plen);
   // Every warp has waited for the last round, so all pushes to this CTA have
-  // landed, and its own have been received.
+  // landed; a peer its own pushes are for stays until it has them.
 }
 
 // CTAs per tree.  Greedy (no slices; a node costs one read of its row and one
@@ -983,6 +1019,7 @@ static adt_status accept_impl(const float* target_logits, const float* target_u,
   p.alen = accept_len;
   p.bonus = bonus_token;
   p.err = info.error_word;
+  p.wait_limit = adt::wait_limit(kWaitLimit) - 1;  // of 1: none (a poll lasts longer than a round)
   p.Vs = vs;
 
   cudaLaunchConfig_t cfg = {};

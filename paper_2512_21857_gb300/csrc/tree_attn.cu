@@ -1639,10 +1639,6 @@ adt_status check_args(const adt_bf16* q, const adt_bf16* k_cache, const adt_bf16
   return ADT_OK;
 }
 
-// Polls before a pipeline wait gives up; 0 = kWaitLimit.  Set only by
-// adt_testing_set_wait_limit.
-uint32_t g_wait_limit = 0;
-
 TcParams make_params(const adt_bf16* q, const int32_t* kv_len, const adt_bf16* k_tree, const adt_bf16* v_tree,
                      const int32_t* parents, const int32_t* node_offsets, int B, int H, int Hkv, int max_kv,
                      int max_nodes, int splits, float scale, adt_bf16* out, float* lse, unsigned* err) {
@@ -1665,19 +1661,13 @@ TcParams make_params(const adt_bf16* q, const int32_t* kv_len, const adt_bf16* k
   prm.out = reinterpret_cast<__nv_bfloat16*>(out);
   prm.lse = lse;
   prm.err = err;
-  const uint32_t lim = __atomic_load_n(&g_wait_limit, __ATOMIC_RELAXED);
-  prm.wait_limit = lim ? lim : kWaitLimit;
+  prm.wait_limit = adt::wait_limit(kWaitLimit);
   return prm;
 }
 
 }  // namespace
 
 extern "C" {
-
-adt_status adt_testing_set_wait_limit(uint32_t polls) {
-  __atomic_store_n(&g_wait_limit, polls, __ATOMIC_RELAXED);
-  return ADT_OK;
-}
 
 size_t adt_tree_attn_workspace_size(int32_t B, int32_t H, int32_t D, int32_t max_nodes,
                                     int32_t max_kv) {
