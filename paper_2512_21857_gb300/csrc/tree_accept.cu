@@ -934,6 +934,23 @@ int cluster_size_for(int V, int B, adt_accept_mode mode) {
   return mode == ADT_ACCEPT_SPEC && V > 32768 && B <= 4 ? 16 : 8;
 }
 
+// The launch limits of instantiation `inst`, once per device and the same
+// whatever call comes first: all the dynamic shared memory a block can have
+// beside the static part, and clusters of 16.
+adt_status configure(void (*kern)(AcceptParams), int inst, const adt::DeviceInfo& info) {
+  static unsigned configured[6][2];  // bit per device (< 64)
+  unsigned& word = configured[inst][(info.device >> 5) & 1];
+  const unsigned bit = 1u << (info.device & 31);
+  if (__atomic_load_n(&word, __ATOMIC_ACQUIRE) & bit) return ADT_OK;
+  cudaFuncAttributes attr;
+  ADT_CUDA_TRY(cudaFuncGetAttributes(&attr, kern));
+  ADT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    info.max_smem_optin - static_cast<int>(attr.sharedSizeBytes)));
+  ADT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  __atomic_fetch_or(&word, bit, __ATOMIC_ACQ_REL);
+  return ADT_OK;
+}
+
 int slice_for(int V, int cs) {
   int vs = (V + cs - 1) / cs;
   return (vs + 3) / 4 * 4;
@@ -978,22 +995,12 @@ static adt_status accept_impl(const float* target_logits, const float* target_u,
   const bool use_df = mode != ADT_ACCEPT_GREEDY && smem_df + sizeof(SampleShared) <= static_cast<size_t>(info.max_smem_optin);
   const size_t smem = mode == ADT_ACCEPT_GREEDY ? 0 : use_df ? smem_df : static_cast<size_t>(vs) * sizeof(float) * nbuf;
   if (smem + sizeof(SampleShared) > static_cast<size_t>(info.max_smem_optin)) return ADT_ERR_UNSUPPORTED;
-  static int configured_smem[64][6];  // largest dynamic smem already allowed, per device and instantiation
-  static int configured_np[64][6];
-  const int dev = info.device & 63;
   auto kern = mode == ADT_ACCEPT_GREEDY ? accept_greedy_kernel
               : mode == ADT_ACCEPT_SPEC
                   ? (use_df ? accept_sample_kernel<true, true> : accept_sample_kernel<false, true>)
                   : (use_df ? accept_sample_kernel<true, false> : accept_sample_kernel<false, false>);
-  const int inst = 2 * static_cast<int>(mode) + (use_df ? 1 : 0);
-  if (configured_smem[dev][inst] < static_cast<int>(smem)) {
-    ADT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    configured_smem[dev][inst] = static_cast<int>(smem);
-  }
-  if (cs > 8 && !configured_np[dev][inst]) {
-    ADT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    configured_np[dev][inst] = 1;
-  }
+  st = configure(kern, 2 * static_cast<int>(mode) + (use_df ? 1 : 0), info);
+  if (st != ADT_OK) return st;
   AcceptParams p;
   p.target = target_logits;
   p.ldt = ld_target;
