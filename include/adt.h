@@ -124,6 +124,12 @@ adt_status adt_testing_set_wait_limit(uint32_t polls);
  * [device] fp32 [n]; out [device] fp64 [n]. */
 adt_status adt_testing_exp_diff(const float* a, const float* b, int32_t n, double* out, void* stream);
 
+/* Testing hook, not for production use: the thread blocks that adt_tree_accept
+ * gives a tree of a call with vocabulary V and B trees, on a device (or the
+ * part of one that a process may use) where `sixteens` clusters of 16 of them
+ * fit at once.  Host only. */
+int32_t adt_testing_accept_cluster(int32_t V, int32_t B, adt_accept_mode mode, int32_t sixteens);
+
 /* ------------------------------------------------------------------------
  * adt_tree_attn - tree-masked attention for one transformer layer.
  *

@@ -25,6 +25,7 @@ DEVERR_BAD_TREE, DEVERR_KV_RANGE, DEVERR_BAD_PATH, DEVERR_TIMEOUT, DEVERR_BAD_IN
 
 EXPORTED = [
     "adt_version", "adt_get_device_error", "adt_status_string", "adt_testing_set_wait_limit", "adt_testing_exp_diff",
+    "adt_testing_accept_cluster",
     "adt_tree_attn_workspace_size", "adt_tree_attn", "adt_tree_attn_noalloc",
     "adt_tree_expand_workspace_size", "adt_tree_expand", "adt_tree_expand_cfg",
     "adt_tree_rerank_workspace_size", "adt_tree_rerank",
@@ -57,6 +58,7 @@ _SIGS = {
     "adt_status_string": ([_I32], ctypes.c_char_p),
     "adt_testing_set_wait_limit": ([ctypes.c_uint32], _I32),
     "adt_testing_exp_diff": ([_P, _P, _I32, _P, _P], _I32),
+    "adt_testing_accept_cluster": ([_I32, _I32, _I32, _I32], _I32),
     "adt_tree_attn_workspace_size": ([_I32] * 5, _SZ),
     "adt_tree_attn": ([_P, _P, _P, _P, _I64, _I64, _P, _P, _P, _P, _I32, _I32, _I32, _I32, _I32, _I32, _F32,
                        _P, _P, _P, _SZ, _P], _I32),

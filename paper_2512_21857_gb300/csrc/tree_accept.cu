@@ -927,11 +927,14 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
 // trees (its exponentials and passes are bound by a cluster's SMs; ten
 // rejections, 8 / 16 CTAs, us: 34.5 / 35.5 at V = 32768, 47.7 / 40.6 at 65536;
 // clusters of 16 for more than about seven trees do not run at once: 49.2 /
-// 68.6 with eight).
-int cluster_size_for(int V, int B, adt_accept_mode mode) {
+// 68.6 with eight).  `sixteens`: the clusters of 16 that fit at once; where a
+// process may use only some of the SMs that can be none, and 8 CTAs serve.
+constexpr int kPortableV = 65536;  // sampling: eight CTAs hold it in double-floats
+
+int cluster_size_for(int V, int B, adt_accept_mode mode, int sixteens) {
   if (mode == ADT_ACCEPT_GREEDY) return V <= 32768 ? 4 : V <= 131072 ? 8 : 16;
-  if (V > 65536) return 16;
-  return mode == ADT_ACCEPT_SPEC && V > 32768 && B <= 4 ? 16 : 8;
+  if (V > kPortableV) return 16;
+  return mode == ADT_ACCEPT_SPEC && V > 32768 && B <= 4 && B <= sixteens ? 16 : 8;
 }
 
 // The launch limits of instantiation `inst`, once per device and the same
@@ -954,6 +957,34 @@ adt_status configure(void (*kern)(AcceptParams), int inst, const adt::DeviceInfo
 int slice_for(int V, int cs) {
   int vs = (V + cs - 1) / cs;
   return (vs + 3) / 4 * 4;
+}
+
+// Clusters of 16 of the SPEC walk that fit on the device at once, with the
+// slices of the largest vocabulary they are a choice for.
+int spec_sixteens(const adt::DeviceInfo& info) {
+  static int cache[64];  // 0 = not queried yet
+  int& slot = cache[info.device & 63];
+  const int v = __atomic_load_n(&slot, __ATOMIC_ACQUIRE);
+  if (v) return v - 1;
+  int num = 0;
+  const auto kern = accept_sample_kernel<true, true>;
+  if (configure(kern, 2 * ADT_ACCEPT_SPEC + 1, info) == ADT_OK) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = 2 * sizeof(float2) * slice_for(kPortableV, 16);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&num, kern, &cfg) != cudaSuccess) num = 0;
+  }
+  if (num == 0) (void)cudaGetLastError();
+  __atomic_store_n(&slot, num + 1, __ATOMIC_RELEASE);
+  return num;
 }
 
 }  // namespace
@@ -987,7 +1018,7 @@ static adt_status accept_impl(const float* target_logits, const float* target_u,
   adt::DeviceInfo info;
   adt_status st = adt::device_info(&info);
   if (st != ADT_OK) return st;
-  const int cs = cluster_size_for(V, B, mode);
+  const int cs = cluster_size_for(V, B, mode, mode == ADT_ACCEPT_SPEC && V <= kPortableV ? spec_sixteens(info) : 0);
   const int vs = slice_for(V, cs);
   const int nbuf = mode == ADT_ACCEPT_SPEC ? 2 : 1;
   // Double-float slices where they fit, fp32 slices otherwise.
@@ -1066,6 +1097,10 @@ adt_status adt_testing_exp_diff(const float* a, const float* b, int32_t n, doubl
   exp_diff_probe_kernel<<<(n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024, 256, 0, adt::as_stream(stream)>>>(a, b, n,
                                                                                                          out);
   return adt::launch_status();
+}
+
+int32_t adt_testing_accept_cluster(int32_t V, int32_t B, adt_accept_mode mode, int32_t sixteens) {
+  return cluster_size_for(V, B, mode, sixteens);
 }
 
 size_t adt_tree_accept_workspace_size(int32_t B, int32_t V) {

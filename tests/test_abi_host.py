@@ -73,6 +73,19 @@ def test_invalid_arguments_rejected_before_launch(lib):
     assert lib.adt_kv_compact_inplace(f, f, f, f, f, f, 8, f, 1, 2, 64, 2, 300, 64, 64, 64, None) == 1
 
 
+def test_acceptance_needs_no_cluster_of_16_up_to_65536_entries(lib):
+    """Clusters of 16 thread blocks are taken up to V = 65536 only where those
+    of all trees fit at once; eight serve any device."""
+    plan = lib.adt_testing_accept_cluster
+    for V in (1, 32768, 32772, 65536):
+        for trees in (1, 4, 5):
+            for mode in (B.ACCEPT_GREEDY, B.ACCEPT_SPEC, B.ACCEPT_SPEC_DET):
+                assert plan(V, trees, mode, 0) <= 8
+                assert plan(V, trees, mode, trees - 1) <= 8
+    assert plan(65536, 4, B.ACCEPT_SPEC, 4) == 16
+    assert plan(65540, 1, B.ACCEPT_SPEC, 0) == 16  # more than eight blocks hold
+
+
 def _run_both(params, grid, accepts):
     ctl_c = B.Controller(*grid, **params)
     op = dict(params)
