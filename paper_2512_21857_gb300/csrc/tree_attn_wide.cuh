@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   __shared__ float2 s_ml[2][kWideRows];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
+  __shared__ int s_bad;
 
   const int rank = blockIdx.x;         // in the cluster, which spans the grid's x extent
   const int h0 = (static_cast<int>(blockIdx.y) - p.prefetch) * p.heads;  // first head of the group
@@ -272,6 +273,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   // kernel).
   if (tid == 0) {
     s_abort = 0;
+    s_bad = 0;
     sm100::mbar_init(sm100::smem_addr(&bars.q_full), 8);
     for (int s = 0; s < NS; ++s) {
       sm100::mbar_init(sm100::smem_addr(&bars.k_full[s]), 1);
@@ -492,24 +494,32 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     sm100::fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) sm100::mbar_arrive(sm100::smem_addr(&bars.q_full));
+    // Parents precede their children; anything else marks the tree malformed:
+    // every CTA of it sees all its nodes (a thread its own copy), and none
+    // writes a row.
+    static_assert(kMaxTreeNodes <= kWideSoftmax, "a thread checks a node");
+    if (tid < n) {
+      const int par = s_par[tid];
+      if ((tid == 0) != (par < 0) || par >= tid) {
+        s_bad = 1;
+        adt::raise_error(p.err, ADT_DEVERR_BAD_TREE);
+      }
+    }
     // While the first products run, where this split has a tree chunk: the
-    // ancestor bits of the tile's nodes.  Parents precede their children; anything else marks the tree malformed
-    // (its rows are left unspecified, and the walk ends there).
+    // ancestor bits of the tile's nodes (of a malformed tree, to where a
+    // parent does not precede its child).
     if (n_tc > 0) {
       static_assert(kWideRows * 2 == kWideSoftmax, "two threads clear a node's bits");
       reinterpret_cast<uint4*>(anc)[tid] = make_uint4(0u, 0u, 0u, 0u);
       wide_softmax_sync();
       if (tid < kWideRows && row0 + tid < n) {
         int j = row0 + tid;
-        bool bad;
         for (;;) {
           atomicOr(&anc[tid][j >> 5], 1u << (j & 31));
           const int par = s_par[j];
-          bad = (j == 0) != (par < 0) || par >= j;
-          if (bad || par < 0) break;
+          if (par < 0 || par >= j) break;
           j = par;
         }
-        if (bad) adt::raise_error(p.err, ADT_DEVERR_BAD_TREE);
       }
       wide_softmax_sync();
     }
@@ -716,7 +726,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 
   if (S == 1) {
     // No other split: the row is final.
-    if (tid < kWideSoftmax && valid) {
+    if (tid < kWideSoftmax && valid && !s_bad) {
       const float inv = __fdividef(1.f, l);
       __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node0 + node) * p.H + h0 + hh) * D + stream * kHalf;
 #pragma unroll
@@ -781,8 +791,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
   sm100::cluster_arrive_release();
   sm100::cluster_wait_acquire();
   auto merge = [&](auto most) {
-    wide_merge<D, decltype(most)::value>(p, reinterpret_cast<const uint8_t*>(rows_out), S, split, tiles, qt, rows_mine,
-                                         r_lo, shift, row0, n, node0, h0);
+    wide_merge<D, decltype(most)::value>(p, reinterpret_cast<const uint8_t*>(rows_out), S, split, tiles, qt,
+                                         s_bad ? 0 : rows_mine, r_lo, shift, row0, n, node0, h0);
   };
   if (S <= 2)
     merge(std::integral_constant<int, 2>());

@@ -92,6 +92,35 @@ def test_wide_bad_tree_sets_device_error():
     assert B.adt_get_device_error() == 0
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("sizes,kv,H,Hkv,max_nodes", [
+    ([150, 70], [700, 300], 20, 20, 256),                  # key splits of two tiles
+    ([64, 33, 5, 17], [1537, 1403, 128, 0], 16, 8, 64),    # two heads a CTA, four splits
+    ([256, 41, 128, 1], [320, 0, 97, 33], 20, 20, 256),    # one split a tile
+])
+def test_wide_bad_tree_is_skipped(sizes, kv, H, Hkv, max_nodes, D):
+    """A malformed tree's rows stay as they were, in every tile and split; the
+    other trees of the call are computed."""
+    case = AttnCase(sizes, kv, H, Hkv, D, seed=sum(sizes) + D, max_depth=10, max_children=39, lmax=max(max(kv), 700))
+    ref, ref_lse = case.run_oracle()
+    n0 = sizes[0]
+    for at, parent in ((n0 - 1, n0 - 1), (1, -1), (0, 0)):
+        good = int(case.tb.parents[at])
+        case.tb.parents[at] = parent
+        out = torch.full((case.ntot, H, D), 7.0, dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((case.ntot, H), 7.0, dtype=torch.float32, device="cuda")
+        B.adt_get_device_error()
+        B.adt_tree_attn(case.q.cuda(), case.kc.cuda(), case.vc.cuda(), i32(kv), case.kt.cuda(), case.vt.cuda(),
+                        i32(case.tb.parents), i32(case.tb.node_offsets), B=case.B, H=H, Hkv=Hkv, D=D,
+                        max_nodes=max_nodes, max_kv=max(kv), softmax_scale=case.scale, out=out, lse=lse,
+                        workspace=B.zeroed_workspace(B.adt_tree_attn_workspace_size(case.B, H, D, max_nodes, max(kv))))
+        assert B.adt_get_device_error() == B.DEVERR_BAD_TREE
+        assert (out[:n0] == 7.0).all() and (lse[:n0] == 7.0).all()
+        assert_attention_close(out[n0:].float().cpu().numpy().astype(np.float64), ref[n0:])
+        assert np.abs(lse[n0:].cpu().numpy() - ref_lse[n0:]).max() < LSE_ATOL
+        case.tb.parents[at] = good
+
+
 def test_wide_wait_that_runs_out_is_reported():
     case = AttnCase([150], [700], 20, 20, 128, seed=6, max_depth=10, max_children=39)
     B.adt_get_device_error()
