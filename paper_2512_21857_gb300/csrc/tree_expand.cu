@@ -760,18 +760,26 @@ struct RerankParams {
 // Rerank of any pool.  The scores are mapped, order kept, to kRerankBins
 // bins over their range; a histogram gives the bin that holds the
 // (n_nodes - 1)-th best, every candidate of a better bin is selected, and the
-// few of that bin are ranked against each other (when they are too many --
-// nearly all scores equal -- a radix select finds the threshold key instead).
-// Node ids follow ascending candidate index (one scan over the warps'
-// counts of all tiles), and node maps, parents and depths stay in shared
-// memory.  Bound by latency: 3.3 us at C = 328, n = 64 (4.6 us when every
-// warp's two largest keys gave the bound), 3.8 us at C = 858, n = 256 (46.3 us
-// with all keys ranked against each other), 6.1 us at C = 6123, n = 256 and
-// 11.8 us at C = 12207 (9.6 and 16.6 us with radix passes over the keys in
-// memory).  M: scores a thread keeps in registers (C <= 1024 M); 0: they are
-// read again where needed.
+// few of that bin are ranked against each other.  More than kRerankFew there
+// -- equal scores, or a few far from the rest that stretch the range -- are
+// binned again over the range of their order keys, as often as it takes (a
+// binning narrows it 1024 times), and by index once they are all equal; in
+// pools too large for registers, up to kRerankList are ranked all the same and
+// a radix select finds the threshold key of more.  Node ids follow ascending
+// candidate index (one scan over the warps' counts of all tiles), and node
+// maps, parents and depths stay in shared memory.
+//
+// Bound by latency.  Scores as grown, us: 3.1 at C = 328, n = 64 (4.5 when every
+// warp's two largest keys gave the bound), 3.7 at C = 858, n = 256 (46 with all
+// keys ranked against each other), 7.0 at C = 6123, n = 256 and 13.6 at C =
+// 12207 (8.9 and 14.5 with radix passes over the keys in memory).  With one
+// score at fp32's lowest value 4.1, 4.6, 8.5 and 13.2, all equal 4.0, 4.1, 8.3
+// and 25 (the crowded bin ranked at once, by a warp a key: 8.9, 29, 8.2 and
+// 13.5, all equal 8.8, 29, 15.6 and 26).  M: scores a thread keeps in registers
+// (C <= 1024 M); 0: they are read again where needed.
 constexpr int kRerankBins = 1024;
-constexpr int kRerankList = 1024;      // candidates of the threshold bin ranked by counting
+constexpr int kRerankList = 1024;      // candidates ranked by counting, at most
+constexpr int kRerankFew = 256;        // ... of scores in registers
 constexpr int kRerankMaxC = 65536;
 constexpr int kRerankMaxNodes = 4096;
 constexpr int kRerankMaxTiles = kRerankMaxC / kRerankThreads;
@@ -779,14 +787,38 @@ constexpr int kRerankRegs = 8;
 
 struct RerankShared {
   int par[kRerankMaxNodes];              // a node's candidate index, then its parent's node id
-  uint64_t list[kRerankList];
+  uint64_t list[kRerankList], nth;
   int hist[kRerankBins];
   int tot[kRerankMaxTiles * 32];         // selected per (tile, warp), then their exclusive prefix
   float fmax[32], fmin[32];
+  uint32_t kmax[32], kmin[32];
   int wsum[32];
   int bin, need, count, nlist, bad;
   adt::RadixScratch rs;
 };
+
+// *nth = the want-th best of the n <= kRerankThreads / T distinct keys: T threads
+// per key, as in rank_select_by.
+template <int T>
+__device__ __forceinline__ void rank_nth_by(const uint64_t* keys, int n, int want, uint64_t* nth) {
+  const int i = threadIdx.x / T, s = threadIdx.x % T;
+  const uint64_t key = i < n ? keys[i] : 0ull;
+  int c = 0;
+#pragma unroll 4
+  for (int o = s; o < n; o += T) c += keys[o] > key ? 1 : 0;
+#pragma unroll
+  for (int off = T / 2; off > 0; off >>= 1) c += __shfl_xor_sync(adt::kFullMask, c, off);
+  if (s == 0 && i < n && c == want - 1) *nth = key;
+}
+
+__device__ __noinline__ void rank_nth(const uint64_t* keys, int n, int want, uint64_t* nth) {
+  if (n <= kRerankThreads / 8)
+    rank_nth_by<8>(keys, n, want, nth);
+  else if (n <= kRerankThreads / 4)
+    rank_nth_by<4>(keys, n, want, nth);
+  else
+    rank_nth_by<1>(keys, n, want, nth);
+}
 
 // Exclusive prefix of one value per thread over the block.
 __device__ __forceinline__ int rerank_block_scan(int v, int* wsum) {
@@ -876,47 +908,105 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankPara
   auto bin_of = [&](float v) -> int {
     return v > -INFINITY ? min(kRerankBins - 1, static_cast<int>((mx - v) * scale)) : kRerankBins - 1;
   };
+  auto find_bin = [&](int want) {  // the bin with the want-th best, from the histogram
+    __syncthreads();
+    const int h = sh.hist[tid];
+    const int before = rerank_block_scan(h, sh.wsum);
+    if (before < want && want <= before + h) {
+      sh.bin = tid;
+      sh.need = want - before;
+      sh.count = h;
+    }
+    __syncthreads();
+  };
   each([&](int, int i, float v) {
     if (i < C) atomicAdd(&sh.hist[bin_of(v)], 1);
   });
-  __syncthreads();
-  {
-    const int h = sh.hist[tid];
-    const int before = rerank_block_scan(h, sh.wsum);
-    if (before < need && need <= before + h) {
-      sh.bin = tid;
-      sh.need = need - before;
-      sh.count = h;
-    }
-  }
-  __syncthreads();
+  find_bin(need);
   const int tbin = sh.bin, tneed = sh.need, tcount = sh.count;
+  auto list_threshold = [&](int n, int want) -> uint64_t {
+    __syncthreads();
+    if (n <= kRerankThreads / 16)
+      rank_nth_by<16>(sh.list, n, want, &sh.nth);
+    else
+      rank_nth(sh.list, n, want, &sh.nth);
+    __syncthreads();
+    return sh.nth;
+  };
   // Bit m of `sel`: candidate tid + 1024 m is selected.
   uint64_t sel = 0ull;
   if (tcount == tneed) {
     each([&](int m, int i, float v) {
       if (i < C && bin_of(v) <= tbin) sel |= 1ull << m;
     });
-  } else if (tcount <= kRerankList) {
+  } else if (tcount <= (M ? kRerankFew : kRerankList)) {
     each([&](int m, int i, float v) {
       if (i >= C) return;
       const int bn = bin_of(v);
       if (bn < tbin) sel |= 1ull << m;
       if (bn == tbin) sh.list[atomicAdd(&sh.nlist, 1)] = adt::select_key(v, static_cast<uint32_t>(i));
     });
-    __syncthreads();
-    // The tneed-th best of the list: warps take keys, lanes count.
-    for (int e = warp; e < tcount; e += kRerankThreads / 32) {
-      const uint64_t ke = sh.list[e];
-      int c = 0;
-      for (int j = lane; j < tcount; j += 32) c += sh.list[j] > ke ? 1 : 0;
-      c = __reduce_add_sync(adt::kFullMask, c);
-      if (lane == 0 && c == tneed - 1) sh.bin = e;  // keys are distinct: one entry has this rank
-    }
-    __syncthreads();
-    const uint64_t thr = sh.list[sh.bin];
+    const uint64_t thr = list_threshold(tcount, tneed);
     each([&](int m, int i, float v) {
       if (i < C && bin_of(v) == tbin && adt::select_key(v, static_cast<uint32_t>(i)) >= thr) sel |= 1ull << m;
+    });
+  } else if constexpr (M > 0) {
+    // Bit m of `in`: the candidate is in the threshold bin.
+    uint64_t in = 0ull;
+    each([&](int m, int i, float v) {
+      if (i >= C) return;
+      const int bn = bin_of(v);
+      if (bn < tbin) sel |= 1ull << m;
+      if (bn == tbin) in |= 1ull << m;
+    });
+    auto each_in = [&](auto f) {
+      each([&](int m, int i, float v) {
+        if ((in >> m) & 1ull) f(m, i, adt::float_order_key(v));
+      });
+    };
+    int want = tneed, count = tcount;
+    do {
+      uint32_t hi = 0u, lo = ~0u;
+      each_in([&](int, int, uint32_t key) {
+        hi = max(hi, key);
+        lo = min(lo, key);
+      });
+      hi = __reduce_max_sync(adt::kFullMask, hi);
+      lo = __reduce_min_sync(adt::kFullMask, lo);
+      if (lane == 0) {
+        sh.kmax[warp] = hi;
+        sh.kmin[warp] = lo;
+      }
+      sh.hist[tid] = 0;
+      __syncthreads();
+      hi = __reduce_max_sync(adt::kFullMask, sh.kmax[lane]);
+      lo = __reduce_min_sync(adt::kFullMask, sh.kmin[lane]);
+      // Equal keys: bins of consecutive indices, one of at most 64 (C <= 65536).
+      const uint32_t range = hi > lo ? hi - lo : static_cast<uint32_t>(C - 1);
+      const int shift = max(0, 22 - __clz(range));
+      auto key_bin = [&](int i, uint32_t key) -> int {
+        return static_cast<int>((hi > lo ? hi - key : static_cast<uint32_t>(i)) >> shift);
+      };
+      each_in([&](int, int i, uint32_t key) { atomicAdd(&sh.hist[key_bin(i, key)], 1); });
+      find_bin(want);
+      const int at = sh.bin;
+      want = sh.need;
+      count = sh.count;
+      each_in([&](int m, int i, uint32_t key) {
+        const int bn = key_bin(i, key);
+        if (bn < at) sel |= 1ull << m;
+        if (bn != at) in &= ~(1ull << m);
+      });
+    } while (count > want && count > kRerankFew);
+    uint64_t thr = 0ull;
+    if (count > want) {
+      each_in([&](int, int i, uint32_t key) {
+        sh.list[atomicAdd(&sh.nlist, 1)] = static_cast<uint64_t>(key) << 32 | (0xffffffffu - static_cast<uint32_t>(i));
+      });
+      thr = list_threshold(count, want);
+    }
+    each_in([&](int m, int i, uint32_t key) {
+      if ((static_cast<uint64_t>(key) << 32 | (0xffffffffu - static_cast<uint32_t>(i))) >= thr) sel |= 1ull << m;
     });
   } else {
     const uint64_t thr = adt::block_topk_threshold<kRerankThreads>(

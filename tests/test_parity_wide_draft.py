@@ -108,6 +108,32 @@ def test_rerank_large_pools(C, n, scores):
 LOWEST = float(np.finfo(np.float32).min)
 
 
+@pytest.mark.parametrize("C,n", [(328, 64), (1024, 256), (6123, 257), (8193, 257)])
+@pytest.mark.parametrize("scores", ["decades", "lowest", "equal", "steps"])
+def test_rerank_scores_that_crowd_a_bin(C, n, scores):
+    """Scores whose range a few of them stretch, so that the rest share a bin,
+    and equal ones: binned again, by value and then by index."""
+    g = np.random.default_rng(C + n)
+    sc = -g.exponential(size=C).astype(np.float32) * 3
+    if scores == "decades":
+        sc[g.choice(C, 30, replace=False)] = -10.0 ** np.arange(3, 33)
+    elif scores == "lowest":
+        sc[::5] = LOWEST
+        sc[3::7] = -np.inf
+        sc[1] = 3e38  # the range leaves fp32
+    elif scores == "equal":
+        sc[:] = -3.0
+        sc[5] = 0.0
+    else:  # neighbouring values around the threshold, 300 of each
+        sc = (np.float32(-1.0) - np.arange(C, dtype=np.float32) // 300 * np.float32(2.0 ** -23)).astype(np.float32)
+        g.shuffle(sc)
+        sc[0] = -1e20
+    got = _rerank(np.arange(C), sc, np.full(C, -1, np.int32), n)
+    order = np.argsort(-sc.astype(np.float64), kind="stable")
+    assert np.array_equal(got["cand_index"][1:], np.sort(order[:n - 1]))
+    assert np.array_equal(got["tokens"][1:], got["cand_index"][1:])
+
+
 @pytest.mark.parametrize("V,k", [(65536, 8), (16384, 39)])  # one row's CTAs: narrow and general instantiation
 @pytest.mark.parametrize("mask", [LOWEST, -np.inf])
 def test_expand_scores_outside_the_range_of_fp32(V, k, mask):
