@@ -903,10 +903,13 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankPara
   mn = -adt::warp_max(-sh.fmin[lane]);
   // Non-increasing in the score (each operation rounds monotonically), so a
   // better bin holds better scores only; equal scores (and +0, -0) share one.
+  // -inf comes last; a NaN, as in the selection keys, first (last with its sign
+  // set).
   const float span = mx - mn;
   const float scale = span > 0.f && span < INFINITY ? (kRerankBins - 1) / span : 0.f;
   auto bin_of = [&](float v) -> int {
-    return v > -INFINITY ? min(kRerankBins - 1, static_cast<int>((mx - v) * scale)) : kRerankBins - 1;
+    if (v > -INFINITY) return min(kRerankBins - 1, static_cast<int>((mx - v) * scale));
+    return __float_as_int(v) < 0 ? kRerankBins - 1 : 0;
   };
   auto find_bin = [&](int want) {  // the bin with the want-th best, from the histogram
     __syncthreads();

@@ -109,10 +109,11 @@ LOWEST = float(np.finfo(np.float32).min)
 
 
 @pytest.mark.parametrize("C,n", [(328, 64), (1024, 256), (6123, 257), (8193, 257)])
-@pytest.mark.parametrize("scores", ["decades", "lowest", "equal", "steps"])
+@pytest.mark.parametrize("scores", ["decades", "lowest", "equal", "steps", "nan"])
 def test_rerank_scores_that_crowd_a_bin(C, n, scores):
     """Scores whose range a few of them stretch, so that the rest share a bin,
-    and equal ones: binned again, by value and then by index."""
+    and equal ones: binned again, by value and then by index.  A NaN ranks
+    first, one with its sign set last."""
     g = np.random.default_rng(C + n)
     sc = -g.exponential(size=C).astype(np.float32) * 3
     if scores == "decades":
@@ -124,12 +125,17 @@ def test_rerank_scores_that_crowd_a_bin(C, n, scores):
     elif scores == "equal":
         sc[:] = -3.0
         sc[5] = 0.0
-    else:  # neighbouring values around the threshold, 300 of each
+    elif scores == "steps":  # neighbouring values around the threshold, 300 of each
         sc = (np.float32(-1.0) - np.arange(C, dtype=np.float32) // 300 * np.float32(2.0 ** -23)).astype(np.float32)
         g.shuffle(sc)
         sc[0] = -1e20
+    else:
+        sc[g.choice(C, 9, replace=False)] = np.nan
+        sc[2] = -np.float32(np.nan)
+        sc[4] = np.inf
     got = _rerank(np.arange(C), sc, np.full(C, -1, np.int32), n)
-    order = np.argsort(-sc.astype(np.float64), kind="stable")
+    order = np.lexsort((np.arange(C), -np.where(np.isnan(sc), 0, sc.astype(np.float64)),
+                        np.where(np.isnan(sc), np.where(np.signbit(sc), 1, -1), 0)))
     assert np.array_equal(got["cand_index"][1:], np.sort(order[:n - 1]))
     assert np.array_equal(got["tokens"][1:], got["cand_index"][1:])
 
