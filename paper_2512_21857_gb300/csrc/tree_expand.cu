@@ -476,13 +476,14 @@ __global__ void __launch_bounds__(kThreads, 1) expand_kernel(const ExpandParams 
   // atomics, no per-element vote).
   const bool large = fabsf(M) >= kLargeRow;
   const float Ml = large ? 0.f : M * kLog2e;
+  const float Ms = large && M != -INFINITY ? M : 0.f;
   auto term = [&](float x) { return ex2_approx(fmaf(x, kLog2e, -Ml)); };
-  auto term_large = [&](float x) { return ex2_approx((x - (M == -INFINITY ? 0.f : M)) * kLog2e); };
+  auto term_any = [&](float x) { return ex2_approx(fmaf(x - Ms, kLog2e, -Ml)); };  // of any share
   float sa[4] = {0.f, 0.f, 0.f, 0.f};
   if constexpr (kRegs) {
     if (large) {
 #pragma unroll
-      for (int e = 0; e < kRegValues; ++e) sa[e % 4] += term_large(xr[e]);
+      for (int e = 0; e < kRegValues; ++e) sa[e % 4] += term_any(xr[e]);
     } else {
 #pragma unroll
       for (int e = 0; e < kRegValues; ++e) sa[e % 4] += term(xr[e]);
@@ -509,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) expand_kernel(const ExpandParams 
         const int i = i0 + u * kThreads;
         if (i < n) {
           const float x = vals[i];
-          sa[u] += large ? term_large(x) : term(x);
+          sa[u] += term_any(x);
           if (x >= B) {
             const unsigned pos = atomicAdd(&s_cnt, 1u);
             if (pos < static_cast<unsigned>(kCandCap)) cand[pos] = adt::select_key(x, static_cast<uint32_t>(t0 + i));
