@@ -341,6 +341,7 @@ struct SampleShared {
   int16_t kid_rep[kBatch];    // 2: that earlier child
   float2 bf[2];               // scalars that warp 0 hands to the block
   int bi[2];
+  int late[3];                // thread 0's, at a batch's start, before the draw and at the end
   int tree_own;               // children of state 0
 };
 
@@ -387,9 +388,11 @@ __device__ __forceinline__ dfl::df resid(dfl::df ep, dfl::df eq, dfl::df B) {
 // parity: a warp pushes for round r + 2 only once round r + 1 is complete, for
 // which every warp of the cluster has pushed after it was done with round r.
 //
-// A wait that runs out raises the error and sets `late` in its thread.  The
-// block barrier that follows every wait, before anything else is pushed, tells
-// the others: the walk ends there, and the CTA pushes no more.
+// A wait that runs out raises the error and sets `late` in its thread.  Thread
+// 0 tells the others across the block barrier that follows every wait, before
+// anything else is pushed: the walk ends there, and the CTA pushes no more.
+// (That thread 0 is not late says that the round is complete.  A vote of the
+// barrier took 0.05 us each.)
 struct Rounds {
   SampleShared* sh;
   unsigned* err;
@@ -586,8 +589,12 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
         ++rd.r;
       }
       if (tid < nb) sh.kid_tok[tid] = tree.tok[tree.kids[base + tid]];
-      if (tid == 0) sh.tree_own = 0;
-      late = __syncthreads_or(rd.late);  // also: this CTA's slices are written
+      if (tid == 0) {
+        sh.tree_own = 0;
+        sh.late[0] = rd.late;
+      }
+      __syncthreads();  // also: this CTA's slices are written
+      late = sh.late[0];
       if (late) break;
       if (tid < nb) {
         const int x = sh.kid_tok[tid];
@@ -689,9 +696,10 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
           if (rd.rank == 0)
             for (int j = lane; j < at; j += 32)
               if (sh.kid_state[j] == 4) adt::raise_error(p.err, ADT_DEVERR_BAD_INDEX);
-          if (lane == 0) sh.bi[0] = at;
+          if (lane == 0) sh.bi[0] = rd.late ? -1 : at;
         }
-        late = __syncthreads_or(rd.late);
+        __syncthreads();
+        late = sh.bi[0] < 0;
         if (late) break;
         if (sh.bi[0] < nb) nxt = tree.kids[base + sh.bi[0]];
       } else {
@@ -740,14 +748,14 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
               break;
             }
             if (lane == 0) {
-              sh.bi[0] = verdict;
+              sh.bi[0] = rd.late ? -1 : verdict;
               sh.bi[1] = j;
               sh.bf[0] = make_float2(nB.hi, nB.lo);
             }
           }
-          late = __syncthreads_or(rd.late);
-          if (late) break;
+          __syncthreads();
           const int verdict = sh.bi[0];
+          late = verdict < 0;
           if (verdict == 1) nxt = tree.kids[base + sh.bi[1]];
           if (verdict != 2) break;
           // The residual mass of the slices at the new B: sum of max(0, e_p -
@@ -824,7 +832,9 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
       // slice and reads it starting at offset t mod its length, wrapping
       // around: at the same step the threads of a half-warp then touch
       // different banks.
-      if (late || __syncthreads_or(rd.late)) break;
+      if (tid == 0) sh.late[1] = rd.late;
+      __syncthreads();
+      if (late || sh.late[1]) break;
       const dfl::df fB{sh.bf[1].x, sh.bf[1].y};
       const int per = (cnt + kThreads - 1) / kThreads;
       const int b0 = min(cnt, tid * per), b1 = min(cnt, b0 + per), len = b1 - b0;
@@ -909,7 +919,9 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
     v = nxt;
     __syncthreads();  // the node's lists are rewritten
   }
-  if (__syncthreads_or(rd.late)) {
+  if (tid == 0) sh.late[2] = rd.late;
+  __syncthreads();
+  if (sh.late[2]) {
     if (rd.rank == 0 && tid == 0) write_skipped(p, b);
     rd.stay();
     return;
