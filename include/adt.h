@@ -126,9 +126,9 @@ adt_status adt_testing_exp_diff(const float* a, const float* b, int32_t n, doubl
 
 /* Testing hook, not for production use: the thread blocks that adt_tree_accept
  * gives a tree of a call with vocabulary V and B trees, on a device (or the
- * part of one that a process may use) where `sixteens` clusters of 16 of them
- * fit at once.  Host only. */
-int32_t adt_testing_accept_cluster(int32_t V, int32_t B, adt_accept_mode mode, int32_t sixteens);
+ * part of one that a process may use) where fit[0] .. fit[3] clusters of 2, 4,
+ * 8 and 16 of them run at once.  Host only. */
+int32_t adt_testing_accept_cluster(int32_t V, int32_t B, adt_accept_mode mode, const int32_t* fit);
 
 /* ------------------------------------------------------------------------
  * adt_tree_attn - tree-masked attention for one transformer layer.

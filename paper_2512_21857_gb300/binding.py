@@ -58,7 +58,7 @@ _SIGS = {
     "adt_status_string": ([_I32], ctypes.c_char_p),
     "adt_testing_set_wait_limit": ([ctypes.c_uint32], _I32),
     "adt_testing_exp_diff": ([_P, _P, _I32, _P, _P], _I32),
-    "adt_testing_accept_cluster": ([_I32, _I32, _I32, _I32], _I32),
+    "adt_testing_accept_cluster": ([_I32, _I32, _I32, ctypes.POINTER(_I32)], _I32),
     "adt_tree_attn_workspace_size": ([_I32] * 5, _SZ),
     "adt_tree_attn": ([_P, _P, _P, _P, _I64, _I64, _P, _P, _P, _P, _I32, _I32, _I32, _I32, _I32, _I32, _F32,
                        _P, _P, _P, _SZ, _P], _I32),

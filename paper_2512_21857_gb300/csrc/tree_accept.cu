@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
       // The warps' totals in index order: a lane scans count / 32 of them.
       // The draw lies in the first warp whose cumulative total passes the
       // target, else in the last one with mass.  (Every warp does this.)
-      const int ne = rd.count() / 32;  // csize * kWarps: 2 to 8
+      const int ne = rd.count() / 32;  // csize * kWarps: 1 to 8
       dfl::df mine{0.f, 0.f};
       for (int k = 0; k < ne; ++k) {
         const float4 t = rd.entries()[lane * ne + k];
@@ -939,14 +939,22 @@ __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptPar
 // trees (its exponentials and passes are bound by a cluster's SMs; ten
 // rejections, 8 / 16 CTAs, us: 34.5 / 35.5 at V = 32768, 47.7 / 40.6 at 65536;
 // clusters of 16 for more than about seven trees do not run at once: 49.2 /
-// 68.6 with eight).  `sixteens`: the clusters of 16 that fit at once; where a
-// process may use only some of the SMs that can be none, and 8 CTAs serve.
-constexpr int kPortableV = 65536;  // sampling: eight CTAs hold it in double-floats
+// 68.6 with eight).  A SPEC CTA fills its SM's registers: fewer a tree where
+// the clusters of more do not all run at once and fewer hold the slices (8 / 4
+// / 2 CTAs, ten rejections, us: 32 trees at V = 4096 75 / 27 / 30, 16 at 16384
+// 59 / 37 / 45, 64 at 16384 144 / 68 / 47, 64 at 32768 168 / 89).  fit[i]: the SPEC
+// clusters of 2 << i that run at once; where a process may use only some of the
+// SMs that can be none of 16.
+constexpr int kSlice = 8192;  // the most entries of a slice of p and one of q in double-floats
 
-int cluster_size_for(int V, int B, adt_accept_mode mode, int sixteens) {
+int cluster_size_for(int V, int B, adt_accept_mode mode, const int* fit) {
   if (mode == ADT_ACCEPT_GREEDY) return V <= 32768 ? 4 : V <= 131072 ? 8 : 16;
-  if (V > kPortableV) return 16;
-  return mode == ADT_ACCEPT_SPEC && V > 32768 && B <= 4 && B <= sixteens ? 16 : 8;
+  if (V > 8 * kSlice) return 16;
+  if (mode == ADT_ACCEPT_SPEC_DET) return 8;
+  if (V > 32768 && B <= 4 && B <= fit[3]) return 16;
+  int cs = 8;
+  for (int i = 2; cs > 2 && B > fit[i] && V <= cs / 2 * kSlice; --i) cs /= 2;
+  return cs;
 }
 
 // The launch limits of instantiation `inst`, once per device and the same
@@ -971,23 +979,23 @@ int slice_for(int V, int cs) {
   return (vs + 3) / 4 * 4;
 }
 
-// Clusters of 16 of the SPEC walk that fit on the device at once, with the
-// slices of the largest vocabulary they are a choice for.
-int spec_sixteens(const adt::DeviceInfo& info) {
-  static int cache[64];  // 0 = not queried yet
-  int& slot = cache[info.device & 63];
+// Clusters of cs CTAs of the SPEC walk that run on the device at once (with the
+// largest slices: a CTA has its SM to itself with smaller ones too).
+int spec_clusters(const adt::DeviceInfo& info, int cs) {
+  static int cache[64][17];  // 0 = not queried yet
+  int& slot = cache[info.device & 63][cs];
   const int v = __atomic_load_n(&slot, __ATOMIC_ACQUIRE);
   if (v) return v - 1;
   int num = 0;
   const auto kern = accept_sample_kernel<true, true>;
   if (configure(kern, 2 * ADT_ACCEPT_SPEC + 1, info) == ADT_OK) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16, 1, 1);
+    cfg.gridDim = dim3(static_cast<unsigned>(cs), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = 2 * sizeof(float2) * slice_for(kPortableV, 16);
+    cfg.dynamicSmemBytes = 2 * sizeof(float2) * kSlice;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(cs);
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -1030,7 +1038,9 @@ static adt_status accept_impl(const float* target_logits, const float* target_u,
   adt::DeviceInfo info;
   adt_status st = adt::device_info(&info);
   if (st != ADT_OK) return st;
-  const int cs = cluster_size_for(V, B, mode, mode == ADT_ACCEPT_SPEC && V <= kPortableV ? spec_sixteens(info) : 0);
+  int fit[4] = {0, 0, 0, 0};
+  for (int i = 0; mode == ADT_ACCEPT_SPEC && i < 4; ++i) fit[i] = spec_clusters(info, 2 << i);
+  const int cs = cluster_size_for(V, B, mode, fit);
   const int vs = slice_for(V, cs);
   const int nbuf = mode == ADT_ACCEPT_SPEC ? 2 : 1;
   // Double-float slices where they fit, fp32 slices otherwise.
@@ -1111,8 +1121,8 @@ adt_status adt_testing_exp_diff(const float* a, const float* b, int32_t n, doubl
   return adt::launch_status();
 }
 
-int32_t adt_testing_accept_cluster(int32_t V, int32_t B, adt_accept_mode mode, int32_t sixteens) {
-  return cluster_size_for(V, B, mode, sixteens);
+int32_t adt_testing_accept_cluster(int32_t V, int32_t B, adt_accept_mode mode, const int32_t* fit) {
+  return cluster_size_for(V, B, mode, fit);
 }
 
 size_t adt_tree_accept_workspace_size(int32_t B, int32_t V) {

@@ -73,17 +73,31 @@ def test_invalid_arguments_rejected_before_launch(lib):
     assert lib.adt_kv_compact_inplace(f, f, f, f, f, f, 8, f, 1, 2, 64, 2, 300, 64, 64, 64, None) == 1
 
 
+def _accept_cluster(lib, V, trees, mode, fit):
+    return lib.adt_testing_accept_cluster(V, trees, mode, (ctypes.c_int32 * 4)(*fit))
+
+
 def test_acceptance_needs_no_cluster_of_16_up_to_65536_entries(lib):
     """Clusters of 16 thread blocks are taken up to V = 65536 only where those
-    of all trees fit at once; eight serve any device."""
-    plan = lib.adt_testing_accept_cluster
+    of all trees run at once; eight serve any device."""
     for V in (1, 32768, 32772, 65536):
         for trees in (1, 4, 5):
             for mode in (B.ACCEPT_GREEDY, B.ACCEPT_SPEC, B.ACCEPT_SPEC_DET):
-                assert plan(V, trees, mode, 0) <= 8
-                assert plan(V, trees, mode, trees - 1) <= 8
-    assert plan(65536, 4, B.ACCEPT_SPEC, 4) == 16
-    assert plan(65540, 1, B.ACCEPT_SPEC, 0) == 16  # more than eight blocks hold
+                for sixteens in (0, trees - 1):
+                    assert _accept_cluster(lib, V, trees, mode, (76, 37, 15, sixteens)) <= 8
+    assert _accept_cluster(lib, 65536, 4, B.ACCEPT_SPEC, (76, 37, 15, 4)) == 16
+    assert _accept_cluster(lib, 65540, 1, B.ACCEPT_SPEC, (0, 0, 0, 0)) == 16  # more than eight blocks hold
+
+
+@pytest.mark.parametrize("V,trees,blocks", [
+    (4096, 15, 8), (4096, 16, 4), (4096, 37, 4), (4096, 38, 2), (4096, 500, 2),
+    (16384, 77, 2), (16388, 77, 4), (32768, 500, 4), (32772, 16, 8), (65536, 500, 8),
+])
+def test_acceptance_splits_many_trees_less(lib, V, trees, blocks):
+    """SPEC: the most thread blocks a tree whose clusters all run at once, of
+    those that hold V in slices of 8192 entries."""
+    assert _accept_cluster(lib, V, trees, B.ACCEPT_SPEC, (76, 37, 15, 7)) == blocks
+    assert _accept_cluster(lib, V, trees, B.ACCEPT_SPEC_DET, (76, 37, 15, 7)) == 8
 
 
 def _run_both(params, grid, accepts):

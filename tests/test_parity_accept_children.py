@@ -10,7 +10,7 @@ import oracle
 from gpu_cases import ensure_built, run_accept_gpu
 from paper_2512_21857_gb300 import binding as B
 from paper_2512_21857_gb300 import synth
-from test_parity_accept_compact import compare
+from test_parity_accept_compact import compare, make_rows
 
 pytestmark = pytest.mark.gpu
 
@@ -101,3 +101,18 @@ def test_cluster_sizes_and_fp32_slices(V):
         tb, target, draft = _star(12, V, V + seed, range(1, 12))
         checked += _check(tb, target, draft, B.ACCEPT_SPEC, seed, margin=1e-9 if V < 200000 else 1e-5) is not None
     assert checked >= 2
+
+
+@pytest.mark.parametrize("trees,V", [(16, 32768), (20, 4099), (40, 4096), (77, 16384), (17, 40000)])
+def test_many_trees(trees, V):
+    """SPEC with 4, 4, 2, 2 and 8 CTAs a tree, in one wave and in two."""
+    for seed in range(V, V + 20):
+        tb = synth.tree_batch([1 + (5 * i) % 13 for i in range(trees)], V, seed, max_depth=4, max_children=6)
+        target, draft = make_rows(tb, V, seed, 0.3)
+        n = len(tb.tokens)
+        ua, us = synth.uniforms(n, seed, "ua"), synth.uniforms(n, seed, "us")
+        res = oracle.tree_accept(target, draft, tb.tokens, tb.parents, tb.node_offsets, B.ACCEPT_SPEC, ua, us)
+        if res["min_margin"] > 1e-9:
+            break
+    assert res["min_margin"] > 1e-9
+    compare(tb, res, *run_accept_gpu(target, draft, tb, B.ACCEPT_SPEC, ua, us))
