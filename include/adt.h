@@ -124,6 +124,14 @@ adt_status adt_testing_set_wait_limit(uint32_t polls);
  * [device] fp32 [n]; out [device] fp64 [n]. */
 adt_status adt_testing_exp_diff(const float* a, const float* b, int32_t n, double* out, void* stream);
 
+/* Testing hook, not for production use: the launch adt_tree_attn makes for
+ * these sizes on the current device.  plan[0]: query rows per thread block (64,
+ * or 128); plan[1]: thread blocks that share the keys of a (tree, query tile,
+ * head), or of all tiles of 128 rows of a (tree, head group); plan[2]: the
+ * clusters a tree's launch has that only prefetch. */
+adt_status adt_testing_attn_plan(int32_t B, int32_t H, int32_t Hkv, int32_t D, int32_t max_nodes, int32_t max_kv,
+                                 int32_t* plan);
+
 /* Testing hook, not for production use: the thread blocks that adt_tree_accept
  * gives a tree of a call with vocabulary V and B trees, on a device (or the
  * part of one that a process may use) where fit[0] .. fit[3] clusters of 2, 4,

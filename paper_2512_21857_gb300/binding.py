@@ -25,7 +25,7 @@ DEVERR_BAD_TREE, DEVERR_KV_RANGE, DEVERR_BAD_PATH, DEVERR_TIMEOUT, DEVERR_BAD_IN
 
 EXPORTED = [
     "adt_version", "adt_get_device_error", "adt_status_string", "adt_testing_set_wait_limit", "adt_testing_exp_diff",
-    "adt_testing_accept_cluster",
+    "adt_testing_attn_plan", "adt_testing_accept_cluster",
     "adt_tree_attn_workspace_size", "adt_tree_attn", "adt_tree_attn_noalloc",
     "adt_tree_expand_workspace_size", "adt_tree_expand", "adt_tree_expand_cfg",
     "adt_tree_rerank_workspace_size", "adt_tree_rerank",
@@ -58,6 +58,7 @@ _SIGS = {
     "adt_status_string": ([_I32], ctypes.c_char_p),
     "adt_testing_set_wait_limit": ([ctypes.c_uint32], _I32),
     "adt_testing_exp_diff": ([_P, _P, _I32, _P, _P], _I32),
+    "adt_testing_attn_plan": ([_I32] * 6 + [ctypes.POINTER(_I32)], _I32),
     "adt_testing_accept_cluster": ([_I32, _I32, _I32, ctypes.POINTER(_I32)], _I32),
     "adt_tree_attn_workspace_size": ([_I32] * 5, _SZ),
     "adt_tree_attn": ([_P, _P, _P, _P, _I64, _I64, _P, _P, _P, _P, _I32, _I32, _I32, _I32, _I32, _I32, _F32,
@@ -169,6 +170,13 @@ def adt_get_device_error(stream=None) -> int:
 def adt_testing_set_wait_limit(polls: int) -> None:
     """Testing hook: polls before the waits of adt_tree_attn and of sampling walks give up (0 = defaults)."""
     _check(lib().adt_testing_set_wait_limit(int(polls)), "adt_testing_set_wait_limit")
+
+
+def adt_testing_attn_plan(B, H, Hkv, D, max_nodes, max_kv):
+    """Testing hook: (query rows a thread block, thread blocks that share the keys, prefetching clusters)."""
+    plan = (_I32 * 3)()
+    _check(lib().adt_testing_attn_plan(B, H, Hkv, D, max_nodes, max_kv, plan), "adt_testing_attn_plan")
+    return tuple(plan)
 
 
 def adt_testing_exp_diff(a, b, out, stream=None) -> None:

@@ -1479,6 +1479,16 @@ int wide_active_clusters(int cluster, int dev) {
   return num;
 }
 
+// The 64-row kernel's prefetching clusters.  At least 2.5 chunks a split: a
+// launch of less is mostly latency.  At D = 64, where a chunk is half the bytes,
+// there is no gain (H = 20, KV 2400: 9.8 and 9.8 us; in the 128-row kernel 12.4
+// and 12.4 us, 192 nodes, KV 693 and 577).
+int tc_prefetch(const TcParams& prm, int D, bool large, bool overlap_previous, int dev) {
+  if (D != 128 || large || !overlap_previous || prm.splits > kMaxClusterSplits) return 0;
+  if (2 * ((prm.max_kv + kChunk - 1) / kChunk + 1) < 5 * prm.splits) return 0;
+  return prefetch_clusters(max_active_clusters(D, large, prm.splits, dev), prm.B * prm.H, prm.B);
+}
+
 template <int D, bool kLarge>
 adt_status launch(TcParams prm, const void* k_cache, const void* v_cache, int64_t sb, int64_t sh, cudaStream_t st,
                   int dev, bool overlap_previous) {
@@ -1500,13 +1510,7 @@ adt_status launch(TcParams prm, const void* k_cache, const void* v_cache, int64_
   if ((s1 = make_rows_map(&tm_vt, prm.vt, D, prm.Hkv)) != ADT_OK) return s1;
   prm.cluster_merge = prm.splits <= kMaxClusterSplits ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
-  // At least 2.5 chunks a split: a launch of less is mostly latency.  At D = 64,
-  // where a chunk is half the bytes, there is no gain (H = 20, KV 2400: 9.8 and
-  // 9.8 us; in the 128-row kernel 12.4 and 12.4 us, 192 nodes, KV 693 and 577).
-  prm.prefetch = 0;
-  if (D == 128 && !kLarge && overlap_previous && prm.cluster_merge &&
-      2 * ((prm.max_kv + kChunk - 1) / kChunk + 1) >= 5 * prm.splits)
-    prm.prefetch = prefetch_clusters(max_active_clusters(D, kLarge, prm.splits, dev), prm.B * prm.H, prm.B);
+  prm.prefetch = tc_prefetch(prm, D, kLarge, overlap_previous, dev);
   cfg.gridDim = dim3(static_cast<unsigned>(prm.splits), static_cast<unsigned>(prm.H + prm.prefetch),
                      static_cast<unsigned>(prm.B * prm.qtiles));
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -1561,6 +1565,27 @@ int wide_heads(const TcParams& prm, int sm_count) {
   return prm.splits <= kMaxClusterSplits && chunks * waves >= kWideChunks * prm.splits ? heads : 0;
 }
 
+// A launch of the 128-row kernel: `heads` (1 or 2) query heads of a kv head per
+// CTA, trees of `tiles` tiles, `groups` (tree, head group) pairs.
+struct WidePlan {
+  int heads, tiles, groups, cluster, prefetch;
+};
+
+template <int D>
+WidePlan wide_plan(const TcParams& prm, int heads, bool overlap_previous, int dev, int sm_count) {
+  WidePlan w;
+  w.heads = heads;
+  w.tiles = (prm.max_tree + kWideRows - 1) / kWideRows;
+  w.groups = prm.B * (prm.H / heads);
+  w.cluster = wide_cluster<D>(sm_count, w.groups, w.tiles, prm.max_kv, dev);
+  w.prefetch = 0;
+  if (D == 128 && overlap_previous) {
+    const int z = w.cluster > 1 ? 1 : w.tiles;  // clusters of one CTA: a tile each
+    w.prefetch = prefetch_clusters(wide_active_clusters<D>(w.cluster, dev), w.groups * z, prm.B * z);
+  }
+  return w;
+}
+
 template <int D>
 adt_status launch_wide(TcParams prm, int heads, const void* k_cache, const void* v_cache, int64_t sb, int64_t sh,
                        cudaStream_t st, int dev, int sm_count, bool overlap_previous) {
@@ -1577,24 +1602,20 @@ adt_status launch_wide(TcParams prm, int heads, const void* k_cache, const void*
   if (s1 != ADT_OK) return s1;
   s1 = make_cache_map(&tm_v, v_cache, D, prm.max_kv, prm.Hkv, prm.B, sh, sb);
   if (s1 != ADT_OK) return s1;
+  ADT_REQUIRE(heads == 1 || heads == 2);  // the kernel's row strides
+  const WidePlan w = wide_plan<D>(prm, heads, overlap_previous, dev, sm_count);
   prm.heads = heads;
   prm.row_stride = kWideRows / heads;
-  const int tiles = (prm.max_tree + kWideRows - 1) / kWideRows;
-  const int groups = prm.B * (prm.H / heads);
-  const int cluster = wide_cluster<D>(sm_count, groups, tiles, prm.max_kv, dev);
+  prm.prefetch = w.prefetch;
   cudaLaunchConfig_t cfg = {};
-  prm.prefetch = 0;
-  if (D == 128 && overlap_previous)
-    prm.prefetch = prefetch_clusters(wide_active_clusters<D>(cluster, dev), groups * (cluster > 1 ? 1 : tiles),
-                                     prm.B * (cluster > 1 ? 1 : tiles));
-  cfg.gridDim = dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(prm.H / heads + prm.prefetch),
-                     static_cast<unsigned>(cluster > 1 ? prm.B : prm.B * tiles));
+  cfg.gridDim = dim3(static_cast<unsigned>(w.cluster), static_cast<unsigned>(prm.H / heads + w.prefetch),
+                     static_cast<unsigned>(w.cluster > 1 ? prm.B : prm.B * w.tiles));
   cfg.blockDim = dim3(kWideThreads, 1, 1);
   cfg.dynamicSmemBytes = WideCfg<D>::kDynSmem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[0].val.clusterDim.x = static_cast<unsigned>(w.cluster);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1] = adt::pdl_attribute();
@@ -1668,6 +1689,33 @@ TcParams make_params(const adt_bf16* q, const int32_t* kv_len, const adt_bf16* k
 }  // namespace
 
 extern "C" {
+
+adt_status adt_testing_attn_plan(int32_t B, int32_t H, int32_t Hkv, int32_t D, int32_t max_nodes, int32_t max_kv,
+                                 int32_t* plan) {
+  ADT_REQUIRE(plan && B >= 1 && Hkv >= 1 && H >= 1 && H % Hkv == 0 && max_kv >= 0);
+  ADT_REQUIRE(max_nodes >= 1 && max_nodes <= kMaxTreeNodes && (D == 64 || D == 128));
+  adt::DeviceInfo info;
+  const adt_status st = adt::device_info(&info);
+  if (st != ADT_OK) return st;
+  const int dev = info.device, Bq = B * qtiles_for(max_nodes);
+  const bool large = max_nodes > kMaxNodes;
+  const int splits = choose_splits(info.sm_count, Bq, H, D, max_kv, dev, large);
+  const TcParams prm = make_params(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, B, H, Hkv, max_kv, max_nodes,
+                                   splits, 1.f, nullptr, nullptr, nullptr);
+  const int heads = wide_heads(prm, info.sm_count);
+  if (heads) {
+    const WidePlan w = D == 128 ? wide_plan<128>(prm, heads, true, dev, info.sm_count)
+                                : wide_plan<64>(prm, heads, true, dev, info.sm_count);
+    plan[0] = kWideRows;
+    plan[1] = w.cluster;
+    plan[2] = w.prefetch;
+  } else {
+    plan[0] = kMaxNodes;
+    plan[1] = splits;
+    plan[2] = tc_prefetch(prm, D, large, true, dev);
+  }
+  return ADT_OK;
+}
 
 size_t adt_tree_attn_workspace_size(int32_t B, int32_t H, int32_t D, int32_t max_nodes,
                                     int32_t max_kv) {

@@ -41,6 +41,16 @@ def test_wide_tiles_match_oracle(sizes, kv, H, Hkv, max_nodes, D):
            max_nodes)
 
 
+def test_wide_more_trees_than_the_launch_orders():
+    """33 trees: past 32 the launch takes them as they come."""
+    sizes = [1 + (7 * i) % 64 for i in range(33)]
+    kv = [(97 * i) % 700 for i in range(33)]
+    assert B.adt_testing_attn_plan(33, 8, 4, 128, 64, 900)[0] == 128
+    case = AttnCase(sizes, kv, 8, 4, 128, seed=33, max_depth=10, max_children=8, lmax=900)
+    got, _, _ = case.run_gpu(max_nodes=64, max_kv=900)
+    assert_attention_close(got, case.run_oracle()[0])
+
+
 @pytest.mark.parametrize("kv", [769, 783, 784, 785, 800, 801, 864, 895])
 def test_wide_prefix_ends(kv):
     """Every kind of end of the last chunk; whatever the cache holds past it (NaN) has no effect."""
