@@ -283,7 +283,8 @@ adt_status adt_tree_expand_cfg(const float* logits_cond, const float* logits_unc
  *
  * cand_token [device] int32 [C]; cand_score [device] fp32 [C];
  * cand_parent [device] int32 [C]; root_token [device] int32 [1].
- * 1 <= n_nodes <= C + 1; C <= 65536; n_nodes <= 4096.
+ * 1 <= n_nodes <= C + 1; C <= 65536; n_nodes <= 4096.  The workspace is checked
+ * (ADT_ERR_WORKSPACE) and not used: its size stays part of this interface.
  * tokens, parents [device] int32 [n_nodes]; cand_index, depth: same or NULL.
  * ------------------------------------------------------------------------ */
 size_t adt_tree_rerank_workspace_size(int32_t C);

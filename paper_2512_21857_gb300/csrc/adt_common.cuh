@@ -68,10 +68,6 @@ inline adt_status launch_status() {
 
 constexpr unsigned kFullMask = 0xffffffffu;
 
-// Programmatic dependent launch: wait until the previous kernel in the
-// stream has completed and its memory is visible (immediate when this launch
-// does not overlap one), then let the next kernel begin launching.  Called
-// before the kernel's first global-memory access.
 // Atomic add at device scope with acquire-release order: writes made
 // visible to the calling thread before it (e.g. through a block barrier)
 // are published with it, and what other threads published with their own
@@ -82,6 +78,10 @@ __device__ __forceinline__ unsigned atomic_add_acq_rel_gpu(unsigned* addr, unsig
   return old;
 }
 
+// Programmatic dependent launch: wait until the previous kernel in the
+// stream has completed and its memory is visible (immediate when this launch
+// does not overlap one), then let the next kernel begin launching.  Called
+// before the kernel's first global-memory access.
 __device__ __forceinline__ void pdl_wait_then_release() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -135,34 +135,6 @@ __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFullMask, v, o));
   return v;
-}
-
-// Block-wide reductions; `scratch` holds >= 32 elements of T.  Every thread
-// receives the result.  Must be called by all threads of the block.
-template <int THREADS, typename T>
-__device__ T block_sum(T v, T* scratch) {
-  static_assert(THREADS % 32 == 0, "");
-  constexpr int W = THREADS / 32;
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  T r = (lane < W) ? scratch[lane] : T(0);
-  r = warp_sum(r);
-  return r;
-}
-
-template <int THREADS>
-__device__ float block_max(float v, float* scratch) {
-  constexpr int W = THREADS / 32;
-  v = warp_max(v);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  float r = (lane < W) ? scratch[lane] : -INFINITY;
-  return warp_max(r);
 }
 
 // Shared memory used by block_topk_threshold.

@@ -55,10 +55,9 @@ struct AcceptParams {
   const int32_t* tokens;
   const int32_t* parents;
   const int32_t* offs;
-  int B, V, max_nodes;
+  int V, max_nodes;
   const float* ua;
   const float* us;
-  int mode;
   float T;
   int use_T;
   int32_t* path;
@@ -1066,12 +1065,10 @@ static adt_status accept_impl(const float* target_logits, const float* target_u,
   p.tokens = tokens;
   p.parents = parents;
   p.offs = node_offsets;
-  p.B = B;
   p.V = V;
   p.max_nodes = max_nodes;
   p.ua = u_accept;
   p.us = u_sample;
-  p.mode = static_cast<int>(mode);
   p.T = temperature;
   p.use_T = mode != ADT_ACCEPT_GREEDY && temperature != 1.0f;
   p.path = path;

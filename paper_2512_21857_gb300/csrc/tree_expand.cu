@@ -1196,6 +1196,8 @@ adt_status adt_tree_expand_cfg(const float* logits_cond, const float* logits_unc
                      keep_idx, next_score, next_id, workspace, workspace_bytes, stream);
 }
 
+// The kernel keeps its scratch in shared memory; callers go on passing what the
+// ABI asks for.
 size_t adt_tree_rerank_workspace_size(int32_t C) {
   if (C < 1) return 0;
   return adt::align_up(static_cast<size_t>(C) * sizeof(int32_t), 256) +
