@@ -21,10 +21,12 @@
 // tests need no further reads.
 //
 // One tree of 64 nodes, ten children of the root, in a graph, before and now:
-// SPEC, all rejected, V = 65536 93.2 -> 40.7 us, V = 16384 51.2 -> 29.7 us;
-// SPEC_DET 23.1 -> 14.0 and 17.6 -> 9.7 us; greedy, four nodes visited, 14.5
-// -> 11.9 and 13.0 -> 10.2 us (one kernel held all three modes and passed
-// every value by a cluster barrier and remote reads).
+// SPEC, all rejected, V = 65536 93.2 -> 40.5 us, V = 16384 51.2 -> 29.5 us;
+// SPEC_DET 23.1 -> 13.9 and 17.6 -> 9.9 us; greedy, four nodes visited, 14.5
+// -> 11.5 and 13.0 -> 9.9 us (one kernel held all three modes and passed
+// every value by a cluster barrier and remote reads).  Of the first, ten
+// rejections are 20.5 us, a root without children (one row's exponentials, the
+// draw) takes 13.8 us and the draft row with its exponentials the rest.
 #include <cooperative_groups.h>
 
 #include "adt_common.cuh"
@@ -503,8 +505,8 @@ __device__ float2 load_rows(const float* trow, const float* trow_u, const float*
 // left after each child do not depend on the walk: their reciprocals are
 // formed at once), and the test u q(x) < p(x) reads u e_q N < (e_p - B e_q) Q.
 // A rejection at V = 16384 / 65536 with 8 CTAs, updating p and q in place with
-// two passes and two exchanges: 3.9 / 7.0 us; this way 2.0 / 3.4 us (2.6 us with 16
-// CTAs).
+// two passes and two exchanges: 3.9 / 7.0 us; this way 1.6 / 2.5 us (2.05 us with
+// 16 CTAs).
 template <bool kDF, bool kSpec>
 __global__ void __launch_bounds__(kThreads) accept_sample_kernel(const AcceptParams p) {
   using SL = Slice<kDF>;

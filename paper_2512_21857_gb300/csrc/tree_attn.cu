@@ -46,9 +46,11 @@
 // the softmax serves every chunk, masks are bit tests on one word per row, the
 // merge is unrolled for the split count's range, and paths off the common one
 // lie behind it (7.4 us at the LlamaGen shape with two softmax copies, 64-bit
-// masks and an eight-way merge inline); the first S product waits for the tensor copies
-// alone, and four threads send the merge's rows (7.3 us without).  One split
-// writes its rows directly (eight ragged trees, 41.9 -> 38.4 us a layer).
+// masks and an eight-way merge inline).  The first S product follows the block
+// barrier after the ancestor walk, but not what the softmax warps do next (the V
+// rows past the tree zeroed, their arrival), and four threads send the merge's
+// rows (7.3 us without these two).  One split writes its rows directly (eight
+// ragged trees, 41.9 -> 38.4 us a layer).
 //
 // Where the 7B launch's 11 us from the dependency wait to the end went before
 // its first chunks were prefetched (cycles at 1.93 GHz): 1500 to the first load,
@@ -732,8 +734,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == kSMmaWarp) {
     // ------------------------------------------------------------ S = Q K^T
     if (lane == 0) {
-      // (Q's copies by the softmax warps end in q_full; a tensor copy needs
-      // nothing of theirs, so the first product goes ahead of the masks.)
+      // (Q's copies by the softmax warps end in q_full, which also follows
+      // their zeroing of V rows; after a tensor copy the first product needs
+      // neither.)
       bool ok = wait_bar(q_tma ? &bars.q_tma : &bars.q_full, 0, &s_abort, p.err, p.wait_limit);
       const uint32_t q_addr = sm100::smem_addr(sQ);
       for (int j = 0; ok && j < nch; ++j) {

@@ -1,13 +1,13 @@
 // Tree attention over 128 query rows at a time: trees of more than 64 nodes,
-// and grouped query heads (several heads of one kv head share a CTA, so that
-// each K and V tile is read once for all of them).  Included by tree_attn.cu,
+// and grouped query heads (two heads of one kv head share a CTA, so that each K
+// and V tile is read once for both).  Included by tree_attn.cu,
 // which holds the 64-row kernel and the shared helpers.
 //
-// A CTA's rows are either 128 consecutive nodes of one head, or `heads` heads
-// of one kv head with row_stride (64 or 32) rows each.  The CTAs of one (tree,
-// head group) form a cluster; a tree's node count, known on the device only,
-// decides how many tiles it has, and the cluster's CTAs are dealt to the tiles
-// as key splits: a call sized for 256 nodes (two tiles) whose tree has 41
+// A CTA's rows are either 128 consecutive nodes of one head (row_stride 128), or
+// two heads of one kv head with 64 rows each (row_stride 64).  The CTAs of one
+// (tree, head group) form a cluster; a tree's node count, known on the device
+// only, decides how many tiles it has, and the cluster's CTAs are dealt to the
+// tiles as key splits: a call sized for 256 nodes (two tiles) whose tree has 41
 // spends all its CTAs on one tile.
 //
 // Warp roles (384 threads): warps 0-3 and 4-7 are two softmax groups that take
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     return;
   }
   const int row0 = qt * kWideRows;
-  const int stride = p.row_stride;  // rows of one head: 128 (one head) or 64
+  const int stride = p.row_stride;  // rows of one head: 128 (one head) or 64 (two)
   const int shift = stride == kWideRows ? 7 : 6;
   const int nrows = p.heads > 1 ? (p.heads - 1) * stride + n : min(n - row0, kWideRows);
   // Chunks of 128 keys: ceil(L / 128) of the prefix, then tree chunks 0 .. qt
