@@ -765,22 +765,27 @@ struct RerankParams {
 // -- equal scores, or a few far from the rest that stretch the range -- are
 // binned again over the range of their order keys, as often as it takes (a
 // binning narrows it 1024 times), and by index once they are all equal; in
-// pools too large for registers, up to kRerankList are ranked all the same and
-// a radix select finds the threshold key of more.  Node ids follow ascending
-// candidate index (one scan over the warps' counts of all tiles), and node
-// maps, parents and depths stay in shared memory.
+// pools too large for registers a radix select finds the threshold key instead,
+// unless all scores are equal.  Pools of up to kRerankDirect are ranked as they
+// are, and a pool that is selected whole is not ranked at all.  Node ids follow
+// ascending candidate index (one scan over the warps' counts of all tiles), and
+// node maps, parents and depths stay in shared memory.
 //
-// Bound by latency.  Scores as grown, us: 3.1 at C = 328, n = 64 (4.5 when every
-// warp's two largest keys gave the bound), 3.7 at C = 858, n = 256 (46 with all
-// keys ranked against each other), 7.0 at C = 6123, n = 256 and 13.6 at C =
-// 12207 (8.9 and 14.5 with radix passes over the keys in memory).  With one
-// score at fp32's lowest value 4.1, 4.6, 8.5 and 13.2, all equal 4.0, 4.1, 8.3
-// and 25 (the crowded bin ranked at once, by a warp a key: 8.9, 29, 8.2 and
-// 13.5, all equal 8.8, 29, 15.6 and 26).  M: scores a thread keeps in registers
-// (C <= 1024 M); 0: they are read again where needed.
+// Bound by latency.  Scores as grown, us: 2.4 at C = 4 to 40 (3.2 by bins), 2.9
+// at C = 100, n = 20 and at C = 328, n = 64 (4.4 when every warp's two largest
+// keys gave the bound), 3.4 at C = 858, n = 256 (46 with all keys ranked against
+// each other), 4.4 at C = 2000, n = 64, 7.3 at C = 6123, n = 256, 13.4 at C =
+// 12207 and 38 at C = 40000, n = 64 (5.1, 9.4, 14.8 and 37.6 with radix passes
+// over the keys in memory).  With one score at fp32's lowest value C = 328, 858,
+// 2000, 6123 and 12207 take 3.8, 4.4, 5.4, 8.8 and 13.2, all equal 3.8, 3.9, 5.3,
+// 8.7 and 18 (the crowded bin ranked at once, by a warp a key: 9.0, 29, 7.1, 8.3
+// and 13.8, all equal 8.9, 29, 11, 15.7 and 26; as before there were bins: 4.4,
+// 46, 6.3, 9.4 and 14.8, all equal 3.6, 46, 10, 15.9 and 24.7).  M: scores a
+// thread keeps in registers (C <= 1024 M), with M = 1 tokens and parents too; 0:
+// they are read again where needed.
 constexpr int kRerankBins = 1024;
-constexpr int kRerankList = 1024;      // candidates ranked by counting, at most
-constexpr int kRerankFew = 256;        // ... of scores in registers
+constexpr int kRerankFew = 256;        // candidates of the threshold bin ranked by counting
+constexpr int kRerankDirect = 128;     // pools ranked by counting as they are
 constexpr int kRerankMaxC = 65536;
 constexpr int kRerankMaxNodes = 4096;
 constexpr int kRerankMaxTiles = kRerankMaxC / kRerankThreads;
@@ -788,7 +793,7 @@ constexpr int kRerankRegs = 8;
 
 struct RerankShared {
   int par[kRerankMaxNodes];              // a node's candidate index, then its parent's node id
-  uint64_t list[kRerankList], nth;
+  uint64_t list[kRerankFew], nth;
   int hist[kRerankBins];
   int tot[kRerankMaxTiles * 32];         // selected per (tile, warp), then their exclusive prefix
   float fmax[32], fmin[32];
@@ -812,87 +817,55 @@ __device__ __forceinline__ void rank_nth_by(const uint64_t* keys, int n, int wan
   if (s == 0 && i < n && c == want - 1) *nth = key;
 }
 
+// n <= kRerankFew.
 __device__ __noinline__ void rank_nth(const uint64_t* keys, int n, int want, uint64_t* nth) {
   if (n <= kRerankThreads / 8)
     rank_nth_by<8>(keys, n, want, nth);
-  else if (n <= kRerankThreads / 4)
-    rank_nth_by<4>(keys, n, want, nth);
   else
-    rank_nth_by<1>(keys, n, want, nth);
+    rank_nth_by<4>(keys, n, want, nth);
+}
+
+// The want-th best of the n keys in the list.  Block-wide.
+__device__ __forceinline__ uint64_t rerank_list_threshold(RerankShared& sh, int n, int want) {
+  __syncthreads();
+  if (n <= kRerankThreads / 16)
+    rank_nth_by<16>(sh.list, n, want, &sh.nth);
+  else
+    rank_nth(sh.list, n, want, &sh.nth);
+  __syncthreads();
+  return sh.nth;
+}
+
+// Inclusive prefix over the warp.
+__device__ __forceinline__ int warp_inclusive(int v) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(adt::kFullMask, v, o);
+    if ((threadIdx.x & 31) >= o) v += y;
+  }
+  return v;
 }
 
 // Exclusive prefix of one value per thread over the block.
 __device__ __forceinline__ int rerank_block_scan(int v, int* wsum) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(adt::kFullMask, incl, o);
-    if (lane >= o) incl += y;
-  }
+  const int incl = warp_inclusive(v);
   if (lane == 31) wsum[warp] = incl;
   __syncthreads();
   const int w = wsum[lane];
-  int wi = w;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(adt::kFullMask, wi, o);
-    if (lane >= o) wi += y;
-  }
-  return __shfl_sync(adt::kFullMask, wi - w, warp) + incl - v;
+  return __shfl_sync(adt::kFullMask, warp_inclusive(w) - w, warp) + incl - v;
 }
 
-template <int M>
-__global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankParams p) {
-  extern __shared__ uint16_t node_of[];  // [C]: a candidate's node id, 0xFFFF if not selected
-  __shared__ RerankShared sh;
+// The n_nodes - 1 best by score bins: bit m of the result is candidate tid + 1024 m.
+// each(f) calls f(m, candidate, score) for every candidate of the thread.
+template <int M, class Each>
+__device__ __forceinline__ uint64_t rerank_by_bins(Each each, const float* cscore, int C, int need, RerankShared& sh) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int need = p.n_nodes - 1, C = p.C;
-  const int tiles = (C + kRerankThreads - 1) / kRerankThreads;
-  sh.hist[tid] = 0;
-  if (tid == 0) {
-    sh.nlist = 0;
-    sh.bad = 0;
-  }
-  adt::pdl_wait_then_release();
-  if (tid == 0) {
-    p.tokens[0] = *p.root;
-    p.parents[0] = -1;
-    if (p.cand_index) p.cand_index[0] = -1;
-    if (p.depth) p.depth[0] = 0;
-    sh.par[0] = -1;
-  }
-  if (need == 0) return;
-  float x[M ? M : 1];
   float mx = -INFINITY, mn = INFINITY;
-  auto see = [&](float v) {
+  each([&](int, int, float v) {
     mx = fmaxf(mx, v);
     mn = v > -INFINITY ? fminf(mn, v) : mn;
-  };
-  if constexpr (M > 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const int i = tid + m * kRerankThreads;
-      x[m] = i < C ? p.cscore[i] : -INFINITY;
-    }
-#pragma unroll
-    for (int m = 0; m < M; ++m) see(x[m]);
-  } else {
-    for (int i = tid; i < C; i += kRerankThreads) see(p.cscore[i]);
-  }
-  // f(m, candidate, score) for every candidate of this thread, tile by tile.
-  auto each = [&](auto f) {
-    if constexpr (M > 0) {
-#pragma unroll
-      for (int m = 0; m < M; ++m)
-        if (m < tiles) f(m, tid + m * kRerankThreads, x[m]);
-    } else {
-      for (int m = 0; m < tiles; ++m) {
-        const int i = tid + m * kRerankThreads;
-        f(m, i, i < C ? p.cscore[i] : -INFINITY);
-      }
-    }
-  };
+  });
   mx = adt::warp_max(mx);
   mn = -adt::warp_max(-mn);
   if (lane == 0) {
@@ -928,33 +901,23 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankPara
   });
   find_bin(need);
   const int tbin = sh.bin, tneed = sh.need, tcount = sh.count;
-  auto list_threshold = [&](int n, int want) -> uint64_t {
-    __syncthreads();
-    if (n <= kRerankThreads / 16)
-      rank_nth_by<16>(sh.list, n, want, &sh.nth);
-    else
-      rank_nth(sh.list, n, want, &sh.nth);
-    __syncthreads();
-    return sh.nth;
-  };
-  // Bit m of `sel`: candidate tid + 1024 m is selected.
   uint64_t sel = 0ull;
   if (tcount == tneed) {
     each([&](int m, int i, float v) {
       if (i < C && bin_of(v) <= tbin) sel |= 1ull << m;
     });
-  } else if (tcount <= (M ? kRerankFew : kRerankList)) {
+  } else if (tcount <= kRerankFew) {
     each([&](int m, int i, float v) {
       if (i >= C) return;
       const int bn = bin_of(v);
       if (bn < tbin) sel |= 1ull << m;
       if (bn == tbin) sh.list[atomicAdd(&sh.nlist, 1)] = adt::select_key(v, static_cast<uint32_t>(i));
     });
-    const uint64_t thr = list_threshold(tcount, tneed);
+    const uint64_t thr = rerank_list_threshold(sh, tcount, tneed);
     each([&](int m, int i, float v) {
       if (i < C && bin_of(v) == tbin && adt::select_key(v, static_cast<uint32_t>(i)) >= thr) sel |= 1ull << m;
     });
-  } else if constexpr (M > 0) {
+  } else if (M > 0 || scale == 0.f) {
     // Bit m of `in`: the candidate is in the threshold bin.
     uint64_t in = 0ull;
     each([&](int m, int i, float v) {
@@ -1007,17 +970,81 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankPara
       each_in([&](int, int i, uint32_t key) {
         sh.list[atomicAdd(&sh.nlist, 1)] = static_cast<uint64_t>(key) << 32 | (0xffffffffu - static_cast<uint32_t>(i));
       });
-      thr = list_threshold(count, want);
+      thr = rerank_list_threshold(sh, count, want);
     }
     each_in([&](int m, int i, uint32_t key) {
       if ((static_cast<uint64_t>(key) << 32 | (0xffffffffu - static_cast<uint32_t>(i))) >= thr) sel |= 1ull << m;
     });
   } else {
     const uint64_t thr = adt::block_topk_threshold<kRerankThreads>(
-        [&](int i) { return adt::select_key(p.cscore[i], static_cast<uint32_t>(i)); }, C, need, &sh.rs);
+        [&](int i) { return adt::select_key(cscore[i], static_cast<uint32_t>(i)); }, C, need, &sh.rs);
     each([&](int m, int i, float v) {
       if (i < C && adt::select_key(v, static_cast<uint32_t>(i)) >= thr) sel |= 1ull << m;
     });
+  }
+  return sel;
+}
+
+template <int M>
+__global__ void __launch_bounds__(kRerankThreads, 1) rerank_kernel(const RerankParams p) {
+  extern __shared__ uint16_t node_of[];  // [C]: a candidate's node id, 0xFFFF if not selected
+  __shared__ RerankShared sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int need = p.n_nodes - 1, C = p.C;
+  const int tiles = (C + kRerankThreads - 1) / kRerankThreads;
+  sh.hist[tid] = 0;
+  if (tid == 0) {
+    sh.nlist = 0;
+    sh.bad = 0;
+  }
+  adt::pdl_wait_then_release();
+  if (tid == 0) {
+    p.tokens[0] = *p.root;
+    p.parents[0] = -1;
+    if (p.cand_index) p.cand_index[0] = -1;
+    if (p.depth) p.depth[0] = 0;
+    sh.par[0] = -1;
+  }
+  if (need == 0) return;
+  float x[M ? M : 1];
+  if constexpr (M > 0) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int i = tid + m * kRerankThreads;
+      x[m] = i < C ? p.cscore[i] : -INFINITY;
+    }
+  }
+  int tok = 0, parent = 0;  // M = 1: the thread's candidate's, loaded with its score
+  if (M == 1 && tid < C) {
+    tok = p.ctok[tid];
+    parent = p.cpar[tid];
+  }
+  // f(m, candidate, score) for every candidate of this thread, tile by tile.
+  auto each = [&](auto f) {
+    if constexpr (M > 0) {
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if (m < tiles) f(m, tid + m * kRerankThreads, x[m]);
+    } else {
+      for (int m = 0; m < tiles; ++m) {
+        const int i = tid + m * kRerankThreads;
+        f(m, i, i < C ? p.cscore[i] : -INFINITY);
+      }
+    }
+  };
+  // Bit m of `sel`: candidate tid + 1024 m is selected.
+  uint64_t sel = 0ull;
+  if (need == C) {
+    each([&](int m, int i, float) {
+      if (i < C) sel |= 1ull << m;
+    });
+  } else if (M == 1 && C <= kRerankDirect) {
+    const uint64_t key = adt::select_key(x[0], static_cast<uint32_t>(tid));
+    if (tid < C) sh.list[tid] = key;
+    const uint64_t thr = rerank_list_threshold(sh, C, need);
+    if (tid < C && key >= thr) sel = 1ull;
+  } else {
+    sel = rerank_by_bins<M>(each, p.cscore, C, need, sh);
   }
   // Node ids in ascending candidate order.
   for (int m = 0; m < tiles; ++m) {
@@ -1025,28 +1052,39 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankPara
     if (lane == 0) sh.tot[m * 32 + warp] = __popc(bal);
   }
   __syncthreads();
-  {
+  int base = 0;  // M = 1: selected in the warps before this one
+  if constexpr (M == 1) {
+    const int t = sh.tot[lane];
+    base = __shfl_sync(adt::kFullMask, warp_inclusive(t) - t, warp);
+  } else {
     const int nt = tiles * 32;  // <= 2 kRerankThreads
     const int a = 2 * tid < nt ? sh.tot[2 * tid] : 0, b = 2 * tid + 1 < nt ? sh.tot[2 * tid + 1] : 0;
     const int before = rerank_block_scan(a + b, sh.wsum);
     if (2 * tid < nt) sh.tot[2 * tid] = before;
     if (2 * tid + 1 < nt) sh.tot[2 * tid + 1] = before + a;
+    __syncthreads();
   }
-  __syncthreads();
   for (int m = 0; m < tiles; ++m) {
     const int i = tid + m * kRerankThreads;
     const bool mine = (sel >> m) & 1ull;
     const unsigned bal = __ballot_sync(adt::kFullMask, mine);
-    const int node = 1 + sh.tot[m * 32 + warp] + __popc(bal & ((1u << lane) - 1u));
+    const int node = 1 + (M == 1 ? base : sh.tot[m * 32 + warp]) + __popc(bal & ((1u << lane) - 1u));
     if (i < C) node_of[i] = mine ? static_cast<uint16_t>(node) : 0xFFFFu;
-    if (mine) sh.par[node] = i;
+    if (mine) sh.par[node] = M == 1 ? parent : i;
+    if (M == 1 && mine) {
+      p.tokens[node] = tok;
+      if (p.cand_index) p.cand_index[node] = i;
+    }
   }
   __syncthreads();
   for (int node = 1 + tid; node <= need; node += kRerankThreads) {
-    const int c = sh.par[node];
-    const int tok = p.ctok[c], pc = p.cpar[c];
-    p.tokens[node] = tok;
-    if (p.cand_index) p.cand_index[node] = c;
+    int pc = sh.par[node];
+    if constexpr (M != 1) {
+      const int c = pc;
+      pc = p.cpar[c];
+      p.tokens[node] = p.ctok[c];
+      if (p.cand_index) p.cand_index[node] = c;
+    }
     int pr = 0;
     if (pc >= 0) {
       const int of = pc < C ? node_of[pc] : 0xFFFF;
@@ -1249,6 +1287,8 @@ adt_status adt_tree_rerank(const int32_t* cand_token, const float* cand_score,
   cfg.dynamicSmemBytes = static_cast<size_t>(C) * sizeof(uint16_t);
   if (C <= kRerankThreads)
     ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<1>, p));
+  else if (C <= 2 * kRerankThreads)
+    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<2>, p));
   else if (C <= kRerankRegs * kRerankThreads)
     ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<kRerankRegs>, p));
   else

@@ -108,11 +108,13 @@ def test_rerank_large_pools(C, n, scores):
 LOWEST = float(np.finfo(np.float32).min)
 
 
-@pytest.mark.parametrize("C,n", [(328, 64), (1024, 256), (6123, 257), (8193, 257)])
+@pytest.mark.parametrize("C,n", [(40, 9), (128, 100), (129, 100), (200, 201), (328, 64), (1024, 256), (2048, 64),
+                                 (2049, 2), (6123, 257), (8193, 257), (40000, 700)])
 @pytest.mark.parametrize("scores", ["decades", "lowest", "equal", "steps", "nan"])
 def test_rerank_scores_that_crowd_a_bin(C, n, scores):
     """Scores whose range a few of them stretch, so that the rest share a bin,
-    and equal ones: binned again, by value and then by index.  A NaN ranks
+    and equal ones: binned again, by value and then by index; pools ranked as
+    they are (up to 128), selected whole, and too large for registers.  A NaN ranks
     first, one with its sign set last."""
     g = np.random.default_rng(C + n)
     sc = -g.exponential(size=C).astype(np.float32) * 3
