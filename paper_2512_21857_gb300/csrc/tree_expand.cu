@@ -774,15 +774,16 @@ struct RerankParams {
 // Bound by latency.  Scores as grown, us: 2.4 at C = 4 to 40 (3.2 by bins), 2.9
 // at C = 100, n = 20 and at C = 328, n = 64 (4.4 when every warp's two largest
 // keys gave the bound), 3.4 at C = 858, n = 256 (46 with all keys ranked against
-// each other), 4.4 at C = 2000, n = 64, 7.3 at C = 6123, n = 256, 13.4 at C =
-// 12207 and 38 at C = 40000, n = 64 (5.1, 9.4, 14.8 and 37.6 with radix passes
-// over the keys in memory).  With one score at fp32's lowest value C = 328, 858,
-// 2000, 6123 and 12207 take 3.8, 4.4, 5.4, 8.8 and 13.2, all equal 3.8, 3.9, 5.3,
-// 8.7 and 18 (the crowded bin ranked at once, by a warp a key: 9.0, 29, 7.1, 8.3
-// and 13.8, all equal 8.9, 29, 11, 15.7 and 26; as before there were bins: 4.4,
-// 46, 6.3, 9.4 and 14.8, all equal 3.6, 46, 10, 15.9 and 24.7).  M: scores a
-// thread keeps in registers (C <= 1024 M), with M = 1 tokens and parents too; 0:
-// they are read again where needed.
+// each other), 4.4 at C = 2000, n = 64, 5.8 at C = 3924, n = 256 (6.1 with eight
+// scores a thread), 7.3 at C = 6123, 13.4 at C = 12207 and 38 at C = 40000, n = 64
+// (5.1, 7.6, 9.4, 14.8 and 37.6 with radix passes over the keys in memory).  With
+// one score at fp32's lowest value C = 328, 858, 2000, 6123 and 12207 take 3.8,
+// 4.4, 5.4, 8.8 and 13.2, all equal 3.8, 3.9, 5.3, 8.7 and 18 (the crowded bin
+// ranked at once, by a warp a key: 9.0, 29, 7.1, 8.3 and 13.8, all equal 8.9, 29,
+// 11, 15.7 and 26; before there were bins: 4.4, 46, 6.3, 9.4 and 14.8, all equal
+// 3.6, 46, 10, 15.9 and 24.7).  M: scores a thread keeps in registers (1, 2, 4 or
+// 8; C <= 1024 M), with M = 1 tokens and parents too; 0: they are read again where
+// needed.
 constexpr int kRerankBins = 1024;
 constexpr int kRerankFew = 256;        // candidates of the threshold bin ranked by counting
 constexpr int kRerankDirect = 128;     // pools ranked by counting as they are
@@ -1289,6 +1290,8 @@ adt_status adt_tree_rerank(const int32_t* cand_token, const float* cand_score,
     ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<1>, p));
   else if (C <= 2 * kRerankThreads)
     ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<2>, p));
+  else if (C <= 4 * kRerankThreads)
+    ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<4>, p));
   else if (C <= kRerankRegs * kRerankThreads)
     ADT_CUDA_TRY(cudaLaunchKernelEx(&cfg, rerank_kernel<kRerankRegs>, p));
   else

@@ -109,7 +109,7 @@ LOWEST = float(np.finfo(np.float32).min)
 
 
 @pytest.mark.parametrize("C,n", [(40, 9), (128, 100), (129, 100), (200, 201), (328, 64), (1024, 256), (2048, 64),
-                                 (2049, 2), (6123, 257), (8193, 257), (40000, 700)])
+                                 (2049, 2), (4096, 300), (6123, 257), (8193, 257), (40000, 700)])
 @pytest.mark.parametrize("scores", ["decades", "lowest", "equal", "steps", "nan"])
 def test_rerank_scores_that_crowd_a_bin(C, n, scores):
     """Scores whose range a few of them stretch, so that the rest share a bin,
